@@ -88,7 +88,7 @@ struct gbi_ctx {
   double mlp_sigma = 0.0;
   int mlp_step = 0;
   bool mlp_ready = false;
-  gbi::Buf nb_cnt, nb_start, nb_tg, nb_sr, nb_scan, cell_of, cell_cnt, cell_start, cell_fill, cell_items, nb_aux;
+  gbi::Buf nb_cnt, nb_start, nb_tg, nb_sr, nb_scan, cell_of, cell_cnt, cell_start, cell_fill, cell_items, nb_aux, nb_slots;
   int nb_pairs = 0, nb_N = 0;
   gbi::Buf mf_F, mf_FR, mf_lab, mf_dO, mf_part, mf_loss;
   int num_sms = 0;

@@ -250,17 +250,17 @@ __device__ __forceinline__ void lab_grad_to_pair(int head, const float* fr, cons
 }
 #endif
 size_t scan_scratch_ints(int n);
-cudaError_t exclusive_scan(const int* in, int* out, int n, int* scratch, cudaStream_t st);
-cudaError_t bbox(int N, const double* R, double* part_dev, double* out_host, cudaStream_t st);
-cudaError_t nb_count_sys(int N, const double* R, const int* sys_of, const int* sys_off, double rc2, int* cnt,
-                         cudaStream_t st);
-cudaError_t nb_fill_sys(int N, const double* R, const int* sys_of, const int* sys_off, double rc2, const int* start,
-                        int* tg, int* sr, cudaStream_t st);
-cudaError_t cells_build(int N, const double* R, const double* box, double side, int* dims, int* cell_of,
-                        int* cell_cnt, int* cell_start, int* cell_fill, int* items, int* scratch, cudaStream_t st);
-cudaError_t nb_cells(int N, const double* R, const double* box, double side, const int* dims, const int* cell_of,
-                     const int* cell_start, const int* cell_cnt, const int* items, double rc2, const int* start,
-                     int* cnt, int* tg, int* sr, int* overflow, cudaStream_t st);
+cudaError_t exclusive_scan(const int* in, int* out, int n, int* total, int* scratch, cudaStream_t st);
+cudaError_t nb_count_sys(int N, const double* R, const int* sys_of, const int* sys_off, int nsys, double rc,
+                         double rc2, int* cnt, cudaStream_t st);
+cudaError_t nb_fill_sys(int N, const double* R, const int* sys_of, const int* sys_off, int nsys, double rc, double rc2,
+                        const int* start, int* tg, int* sr, cudaStream_t st);
+int nb_cell_bits(int N);
+size_t nb_slot_ints(int N);
+cudaError_t nb_search(int N, const double* R, double rc, double rc2, int* cell_of, int* rank, int* cell_cnt,
+                      int* cell_start, void* rec, int* scratch, int* cnt, int* slots, int* overflow,
+                      cudaStream_t st);
+cudaError_t nb_pack(int N, const int* start, const int* cnt, const int* slots, int* tg, int* sr, cudaStream_t st);
 cudaError_t features(int P, const double* R, const double* p, const int* tg, const int* sr, double a, float* F,
                      float* FR, cudaStream_t st);
 size_t packed_bytes();

@@ -81,12 +81,55 @@ __global__ void k_scan_add(int* __restrict__ out, int n, const int* __restrict__
 
 size_t scan_scratch_ints(int n) { return (size_t)((n + 1023) / 1024) + 1; }
 
-cudaError_t exclusive_scan(const int* in, int* out, int n, int* scratch, cudaStream_t st) {
+// Up to this many counts one kernel scans: every block adds up all the counts before its own
+// chunk itself (L2 reads, at most 1 MB a block) instead of waiting for the other blocks or for
+// two more launches.  n = 10^5: one launch against three (9 us).
+constexpr int kScanOne = 1 << 18;
+
+__device__ __forceinline__ int block_sum_1024(int v, int* s_warp) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) s_warp[w] = v;
+  __syncthreads();
+  int t = s_warp[lane];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  __syncthreads();
+  return t;
+}
+
+__global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ in, int* __restrict__ out, int n,
+                                                   int* __restrict__ total_out) {
+  __shared__ int s_warp[32];
+  const int n4 = blockIdx.x * 256;   // int4s before this chunk
+  const int4* in4 = reinterpret_cast<const int4*>(in);
+  int acc = 0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n4; i += 1024) {
+    const int4 v = in4[i];
+    acc += (v.x + v.y) + (v.z + v.w);
+  }
+  const int before = block_sum_1024(acc, s_warp);
+  const int i = blockIdx.x * 1024 + threadIdx.x;
+  const int v = i < n ? in[i] : 0;
+  int total = 0;
+  const int e = block_exclusive_scan_1024(v, s_warp, total);
+  if (i < n) out[i] = before + e;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total_out = before + total;
+}
+
+// out = exclusive scan of in (16-byte aligned), *total = its sum
+cudaError_t exclusive_scan(const int* in, int* out, int n, int* total, int* scratch, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int chunks = (n + 1023) / 1024;
+  if (n <= kScanOne) {
+    k_scan_one<<<chunks, 1024, 0, st>>>(in, out, n, total);
+    return cudaGetLastError();
+  }
   if (chunks > 1024) return cudaErrorInvalidValue;
   k_scan_chunks<<<chunks, 1024, 0, st>>>(in, out, n, scratch);
-  k_scan_sums<<<1, 1024, 0, st>>>(scratch, chunks, scratch + chunks);
+  k_scan_sums<<<1, 1024, 0, st>>>(scratch, chunks, total);
   k_scan_add<<<chunks, 1024, 0, st>>>(out, n, scratch);
   return cudaGetLastError();
 }
@@ -103,17 +146,13 @@ __device__ __forceinline__ double dist2(const double* a, const double* b) {
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-// small systems (or one system small enough for O(N^2)): scan the whole system
+// batches of small systems: one thread per target scans its system
 __global__ void k_nb_sys(int N, const double* __restrict__ R, const int* __restrict__ sys_of,
                          const int* __restrict__ sys_off, double rc2, const int* __restrict__ start,
                          int* __restrict__ cnt, int* __restrict__ tg, int* __restrict__ sr) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
-  int lo = 0, hi = N;
-  if (sys_of != nullptr) {
-    lo = sys_off[sys_of[n]];
-    hi = sys_off[sys_of[n] + 1];
-  }
+  const int lo = sys_off[sys_of[n]], hi = sys_off[sys_of[n] + 1];
   const double* rn = R + 3 * (size_t)n;
   int c = 0;
   const int base = start != nullptr ? start[n] : 0;
@@ -130,120 +169,184 @@ __global__ void k_nb_sys(int N, const double* __restrict__ R, const int* __restr
   if (start == nullptr) cnt[n] = c;
 }
 
-struct CellGrid {
-  double lo[3];
-  double inv;      // 1 / cell side
-  int dim[3];
+// Distance test in FP32 with a margin.  For a target whose largest coordinate is |x| the
+// FP32 centres of any pair closer than rc carry an error of at most M 2^-24 each, M = |x| + rc,
+// so the FP32 squared distance is off by less than marg = rc M 2^-20 + M^2 2^-44 + 4e-6 rc^2:
+// below rc^2 - marg the pair is inside, above rc^2 + marg it is outside, and only in between
+// (a few pairs in 10^5; NaN too) does the FP64 test of the definition decide.  FP64 costs 64
+// times FP32 here: with it on every candidate a pass over 10^5 spheres took 250 us.
+struct NearTest {
+  float lo, hi;
+  __device__ __forceinline__ NearTest(float x, float y, float z, double rc) {
+    const float r = float(rc);
+    if (!(rc > 1e-15 && rc < 1e15)) {   // squares leave the FP32 range: FP64 decides
+      lo = -INFINITY;
+      hi = INFINITY;
+      return;
+    }
+    const float M = fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z))) + r;
+    const float marg = r * M * 9.5367432e-7f + M * M * 5.6843419e-14f + 4e-6f * r * r;
+    lo = r * r - marg;
+    hi = r * r + marg;
+  }
+  // 1: inside, 0: outside, -1: undecided
+  __device__ __forceinline__ int operator()(float dx, float dy, float dz) const {
+    const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+    return d2 < lo ? 1 : (d2 > hi ? 0 : -1);
+  }
 };
 
-__device__ __forceinline__ int cell_coord(double x, double lo, double inv, int dim) {
-  int c = int(floor((x - lo) * inv));
-  return c < 0 ? 0 : (c >= dim ? dim - 1 : c);
+// one system small enough for O(N^2), or a batch of larger systems: one warp per target scans
+// its system 32 sources at a time; the ballot keeps the sources in order
+__global__ void k_nb_warp(int N, const double* __restrict__ R, const int* __restrict__ sys_of,
+                          const int* __restrict__ sys_off, double rc, double rc2, const int* __restrict__ start,
+                          int* __restrict__ cnt, int* __restrict__ tg, int* __restrict__ sr) {
+  const int n = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (n >= N) return;
+  int lo = 0, hi = N;
+  if (sys_of != nullptr) {
+    lo = sys_off[sys_of[n]];
+    hi = sys_off[sys_of[n] + 1];
+  }
+  const double* rn = R + 3 * (size_t)n;
+  const float x = float(rn[0]), y = float(rn[1]), z = float(rn[2]);
+  const NearTest test(x, y, z, rc);
+  int c = start != nullptr ? start[n] : 0;
+  for (int b = lo; b < hi; b += 32) {
+    const int m = b + lane;
+    bool in = false;
+    if (m < hi && m != n) {
+      const double* rm = R + 3 * (size_t)m;
+      const int t = test(x - float(rm[0]), y - float(rm[1]), z - float(rm[2]));
+      in = t > 0 || (t < 0 && dist2(rn, rm) < rc2);
+    }
+    const unsigned int mask = __ballot_sync(0xffffffffu, in);
+    if (start != nullptr && in) {
+      const int k = c + __popc(mask & ((1u << lane) - 1u));
+      tg[k] = n;
+      sr[k] = m;
+    }
+    c += __popc(mask);
+  }
+  if (start == nullptr && lane == 0) cnt[n] = c;
 }
 
+// Cells of side slightly above rc folded onto a table of 2^(lx + ly + lz) buckets (cell
+// coordinates modulo the powers of two, each at least 4 so that a cell's 27 neighbours fall
+// into 27 different buckets).  No bounding box is needed, the table has about one bucket per
+// sphere whatever the extent, and far cells that share a bucket only add candidates.
+struct CellGrid {
+  double inv;      // 1 / cell side
+  int lx, ly, lz;
+};
+
+__device__ __forceinline__ int cell_coord(double x, double inv, int lg) {
+  return int((long long)floor(x * inv) & ((1ll << lg) - 1));
+}
+
+// the bucket of every sphere and its place among the bucket's spheres (in order of arrival:
+// the neighbour lists are sorted afterwards)
 __global__ void k_cell_count(int N, const double* __restrict__ R, CellGrid g, int* __restrict__ cell_of,
-                             int* __restrict__ cell_cnt) {
+                             int* __restrict__ rank, int* __restrict__ cell_cnt) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   const double* r = R + 3 * (size_t)n;
-  const int cx = cell_coord(r[0], g.lo[0], g.inv, g.dim[0]);
-  const int cy = cell_coord(r[1], g.lo[1], g.inv, g.dim[1]);
-  const int cz = cell_coord(r[2], g.lo[2], g.inv, g.dim[2]);
-  const int c = (cz * g.dim[1] + cy) * g.dim[0] + cx;
+  const int c = (((cell_coord(r[2], g.inv, g.lz) << g.ly) + cell_coord(r[1], g.inv, g.ly)) << g.lx) +
+                cell_coord(r[0], g.inv, g.lx);
   cell_of[n] = c;
-  atomicAdd(&cell_cnt[c], 1);
+  rank[n] = atomicAdd(&cell_cnt[c], 1);
 }
 
-// slot order within a cell depends on timing; the neighbour lists are sorted afterwards
-__global__ void k_cell_fill(int N, const int* __restrict__ cell_of, const int* __restrict__ cell_start,
-                            int* __restrict__ cell_fill, int* __restrict__ items) {
+// records (FP32 centre, index) in bucket order, read contiguously by the search
+__global__ void k_cell_fill(int N, const double* __restrict__ R, const int* __restrict__ cell_of,
+                            const int* __restrict__ rank, const int* __restrict__ cell_start,
+                            float4* __restrict__ rec) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
-  const int c = cell_of[n];
-  items[cell_start[c] + atomicAdd(&cell_fill[c], 1)] = n;
+  const double* r = R + 3 * (size_t)n;
+  rec[cell_start[cell_of[n]] + rank[n]] = make_float4(float(r[0]), float(r[1]), float(r[2]), __int_as_float(n));
 }
 
 constexpr int kMaxNb = 64;   // neighbours kept per sphere in the cell-list path
 
-__global__ void k_nb_cells(int N, const double* __restrict__ R, CellGrid g, const int* __restrict__ cell_of,
-                           const int* __restrict__ cell_start, const int* __restrict__ cell_cnt,
-                           const int* __restrict__ items, double rc2, const int* __restrict__ start,
-                           int* __restrict__ cnt, int* __restrict__ tg, int* __restrict__ sr,
-                           int* __restrict__ overflow) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  const double* rn = R + 3 * (size_t)n;
+// Neighbours of every sphere, in no particular order, into its row of kMaxNb slots, and their
+// number.  One thread per record in bucket order, so the lanes of a warp walk the same buckets
+// (the three buckets along x are one range unless they wrap); the ends of the nine rows'
+// ranges are loaded together ahead of the walk.  One search instead of a counting and a filling
+// one: the slots' memory traffic (~30 bytes a sphere) is far below a second search.  N = 10^5 at
+// volume fraction 0.1 (ncu): 34 us and 8 us for k_nb_pack (two FP64 searches with a local array
+// took 250 us each; with each range loaded as it is walked 51 us): latency of the dependent
+// loads with 20 warps per SM.
+__global__ void __launch_bounds__(128) k_nb_search(int N, const double* __restrict__ R, CellGrid g,
+                                                   const int* __restrict__ cell_of,
+                                                   const int* __restrict__ cell_start,
+                                                   const float4* __restrict__ rec, double rc, double rc2,
+                                                   int* __restrict__ cnt, int* __restrict__ slots,
+                                                   int* __restrict__ overflow) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= N) return;
+  const float4 q = rec[t];
+  const int n = __float_as_int(q.w);
   const int c = cell_of[n];
-  const int cx = c % g.dim[0], cy = (c / g.dim[0]) % g.dim[1], cz = c / (g.dim[0] * g.dim[1]);
-  int nb[kMaxNb];
+  const int mx = (1 << g.lx) - 1, my = (1 << g.ly) - 1, mz = (1 << g.lz) - 1;
+  const int cx = c & mx, cy = (c >> g.lx) & my, cz = c >> (g.lx + g.ly);
+  const NearTest test(q.x, q.y, q.z, rc);
+  int* row = slots + (size_t)n * kMaxNb;
   int k = 0;
-  for (int dz = -1; dz <= 1; ++dz) {
-    const int z = cz + dz;
-    if (z < 0 || z >= g.dim[2]) continue;
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int y = cy + dy;
-      if (y < 0 || y >= g.dim[1]) continue;
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int x = cx + dx;
-        if (x < 0 || x >= g.dim[0]) continue;
-        const int cc = (z * g.dim[1] + y) * g.dim[0] + x;
-        const int b = cell_start[cc], e = b + cell_cnt[cc];
-        for (int i = b; i < e; ++i) {
-          const int m = items[i];
-          if (m == n || !(dist2(rn, R + 3 * (size_t)m) < rc2)) continue;
-          if (k < kMaxNb) nb[k] = m;
-          ++k;
-        }
-      }
+  auto scan = [&](int b, int e) {
+#pragma unroll 2
+    for (int i = b; i < e; ++i) {
+      const float4 s = rec[i];
+      const int in = test(q.x - s.x, q.y - s.y, q.z - s.z);
+      if (in == 0 || i == t) continue;
+      const int m = __float_as_int(s.w);
+      if (in < 0 && !(dist2(R + 3 * (size_t)n, R + 3 * (size_t)m) < rc2)) continue;
+      if (k < kMaxNb) row[k] = m;
+      ++k;
+    }
+  };
+  // the buckets cx - 1, cx, cx + 1 of a row: one range, and the bucket at the other end of the
+  // row when one of them wraps
+  const int x0 = cx > 0 ? cx - 1 : 0, x1 = cx < mx ? cx + 2 : mx + 1;
+  const int xw = cx == 0 ? mx : (cx == mx ? 0 : -1);
+  int rb[9], re[9];
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    const int r = ((((cz + j / 3 - 1) & mz) << g.ly) + ((cy + j % 3 - 1) & my)) << g.lx;
+    rb[j] = cell_start[r + x0];
+    re[j] = cell_start[r + x1];
+  }
+#pragma unroll
+  for (int j = 0; j < 9; ++j) scan(rb[j], re[j]);
+  if (xw >= 0) {
+    for (int j = 0; j < 9; ++j) {
+      const int r = ((((cz + j / 3 - 1) & mz) << g.ly) + ((cy + j % 3 - 1) & my)) << g.lx;
+      scan(cell_start[r + xw], cell_start[r + xw + 1]);
     }
   }
   if (k > kMaxNb) {
     atomicExch(overflow, 1);
     k = kMaxNb;
   }
-  if (start == nullptr) {
-    cnt[n] = k;
-    return;
-  }
-  // insertion sort by source index: the list no longer depends on the cell slot order
-  for (int i = 1; i < k; ++i) {
-    const int v = nb[i];
-    int j = i - 1;
-    while (j >= 0 && nb[j] > v) {
-      nb[j + 1] = nb[j];
-      --j;
-    }
-    nb[j + 1] = v;
-  }
-  const int base = start[n];
-  for (int i = 0; i < k; ++i) {
-    tg[base + i] = n;
-    sr[base + i] = nb[i];
-  }
+  cnt[n] = k;
 }
 
-__global__ void k_bbox(int N, const double* __restrict__ R, double* __restrict__ part) {
-  __shared__ double s[6][256];
-  double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x)
-    for (int d = 0; d < 3; ++d) {
-      mn[d] = fmin(mn[d], R[3 * (size_t)n + d]);
-      mx[d] = fmax(mx[d], R[3 * (size_t)n + d]);
-    }
-  for (int d = 0; d < 3; ++d) {
-    s[d][threadIdx.x] = mn[d];
-    s[3 + d][threadIdx.x] = mx[d];
+// The slots' neighbours into the pair list, sorted by source within a target: eight lanes per
+// target, each placing its entries by counting the smaller ones in the row
+__global__ void k_nb_pack(int N, const int* __restrict__ start, const int* __restrict__ cnt,
+                          const int* __restrict__ slots, int* __restrict__ tg, int* __restrict__ sr) {
+  const int gt = blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = gt >> 3, l = gt & 7;
+  if (n >= N) return;
+  const int c = cnt[n], base = start[n];
+  const int* row = slots + (size_t)n * kMaxNb;
+  for (int i = l; i < c; i += 8) {
+    const int m = row[i];
+    int k = base;
+    for (int j = 0; j < c; ++j) k += row[j] < m ? 1 : 0;
+    tg[k] = n;
+    sr[k] = m;
   }
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-      for (int d = 0; d < 3; ++d) {
-        s[d][threadIdx.x] = fmin(s[d][threadIdx.x], s[d][threadIdx.x + o]);
-        s[3 + d][threadIdx.x] = fmax(s[3 + d][threadIdx.x], s[3 + d][threadIdx.x + o]);
-      }
-    __syncthreads();
-  }
-  if (threadIdx.x < 6) part[blockIdx.x * 6 + threadIdx.x] = s[threadIdx.x][0];
 }
 
 // ---------------------------------------------------------------------------------
@@ -837,69 +940,65 @@ cudaError_t adam(float* th, float* m, float* v, const float* g, int t, double lr
 // neighbour-list driver
 // ---------------------------------------------------------------------------------
 
-cudaError_t bbox(int N, const double* R, double* part_dev, double* out_host, cudaStream_t st) {
-  const int blocks = N < 256 * 64 ? (N + 255) / 256 : 64;
-  k_bbox<<<blocks, 256, 0, st>>>(N, R, part_dev);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  double tmp[64 * 6];
-  e = cudaMemcpyAsync(tmp, part_dev, sizeof(double) * 6 * blocks, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return e;
-  for (int d = 0; d < 3; ++d) {
-    out_host[d] = 1e300;
-    out_host[3 + d] = -1e300;
-  }
-  for (int b = 0; b < blocks; ++b)
-    for (int d = 0; d < 3; ++d) {
-      out_host[d] = fmin(out_host[d], tmp[6 * b + d]);
-      out_host[3 + d] = fmax(out_host[3 + d], tmp[6 * b + 3 + d]);
-    }
-  return cudaSuccess;
-}
+// systems of this many spheres on average are scanned by a warp per target
+constexpr int kNbWarpMean = 16;
 
-cudaError_t nb_count_sys(int N, const double* R, const int* sys_of, const int* sys_off, double rc2, int* cnt,
-                         cudaStream_t st) {
-  k_nb_sys<<<(N + 127) / 128, 128, 0, st>>>(N, R, sys_of, sys_off, rc2, nullptr, cnt, nullptr, nullptr);
+static cudaError_t nb_scan_systems(int N, const double* R, const int* sys_of, const int* sys_off, int nsys, double rc,
+                                   double rc2, const int* start, int* cnt, int* tg, int* sr, cudaStream_t st) {
+  if (sys_of != nullptr && N < (long long)kNbWarpMean * nsys)
+    k_nb_sys<<<(N + 127) / 128, 128, 0, st>>>(N, R, sys_of, sys_off, rc2, start, cnt, tg, sr);
+  else
+    k_nb_warp<<<(N + 3) / 4, 128, 0, st>>>(N, R, sys_of, sys_off, rc, rc2, start, cnt, tg, sr);
   return cudaGetLastError();
 }
 
-cudaError_t nb_fill_sys(int N, const double* R, const int* sys_of, const int* sys_off, double rc2, const int* start,
-                        int* tg, int* sr, cudaStream_t st) {
-  k_nb_sys<<<(N + 127) / 128, 128, 0, st>>>(N, R, sys_of, sys_off, rc2, start, nullptr, tg, sr);
-  return cudaGetLastError();
+cudaError_t nb_count_sys(int N, const double* R, const int* sys_of, const int* sys_off, int nsys, double rc,
+                         double rc2, int* cnt, cudaStream_t st) {
+  return nb_scan_systems(N, R, sys_of, sys_off, nsys, rc, rc2, nullptr, cnt, nullptr, nullptr, st);
 }
 
-cudaError_t cells_build(int N, const double* R, const double* box, double side, int* dims, int* cell_of,
-                        int* cell_cnt, int* cell_start, int* cell_fill, int* items, int* scratch, cudaStream_t st) {
+cudaError_t nb_fill_sys(int N, const double* R, const int* sys_of, const int* sys_off, int nsys, double rc, double rc2,
+                        const int* start, int* tg, int* sr, cudaStream_t st) {
+  return nb_scan_systems(N, R, sys_of, sys_off, nsys, rc, rc2, start, nullptr, tg, sr, st);
+}
+
+// log2 of the buckets of N spheres: about one each, between 4 x 4 x 4 and 2^20
+int nb_cell_bits(int N) {
+  int b = 6;
+  while (b < 20 && (1 << b) < N) ++b;
+  return b;
+}
+
+size_t nb_slot_ints(int N) { return (size_t)N * kMaxNb; }
+
+// bucket lists and the neighbours of every sphere (counts and slots); cell_start has one entry
+// more than there are buckets
+cudaError_t nb_search(int N, const double* R, double rc, double rc2, int* cell_of, int* rank, int* cell_cnt,
+                      int* cell_start, void* rec, int* scratch, int* cnt, int* slots, int* overflow,
+                      cudaStream_t st) {
+  const int bits = nb_cell_bits(N);
   CellGrid g;
-  for (int d = 0; d < 3; ++d) {
-    g.lo[d] = box[d];
-    g.dim[d] = dims[d];
-  }
-  g.inv = 1.0 / side;
-  const int nc = dims[0] * dims[1] * dims[2];
+  g.lx = (bits + 2) / 3;
+  g.ly = (bits + 1) / 3;
+  g.lz = bits / 3;
+  // the side exceeds rc by more than the rounding of x / side, so that spheres closer than rc
+  // are never two cells apart
+  g.inv = 1.0 / (rc * (1.0 + 1.0 / 1048576.0));
+  const int nc = 1 << bits;
   cudaError_t e = cudaMemsetAsync(cell_cnt, 0, sizeof(int) * nc, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(cell_fill, 0, sizeof(int) * nc, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(overflow, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_cell_count<<<(N + 255) / 256, 256, 0, st>>>(N, R, g, cell_of, cell_cnt);
-  e = exclusive_scan(cell_cnt, cell_start, nc, scratch, st);
+  k_cell_count<<<(N + 255) / 256, 256, 0, st>>>(N, R, g, cell_of, rank, cell_cnt);
+  e = exclusive_scan(cell_cnt, cell_start, nc, cell_start + nc, scratch, st);
   if (e != cudaSuccess) return e;
-  k_cell_fill<<<(N + 255) / 256, 256, 0, st>>>(N, cell_of, cell_start, cell_fill, items);
+  k_cell_fill<<<(N + 255) / 256, 256, 0, st>>>(N, R, cell_of, rank, cell_start, static_cast<float4*>(rec));
+  k_nb_search<<<(N + 127) / 128, 128, 0, st>>>(N, R, g, cell_of, cell_start, static_cast<const float4*>(rec), rc, rc2,
+                                               cnt, slots, overflow);
   return cudaGetLastError();
 }
 
-cudaError_t nb_cells(int N, const double* R, const double* box, double side, const int* dims, const int* cell_of,
-                     const int* cell_start, const int* cell_cnt, const int* items, double rc2, const int* start,
-                     int* cnt, int* tg, int* sr, int* overflow, cudaStream_t st) {
-  CellGrid g;
-  for (int d = 0; d < 3; ++d) {
-    g.lo[d] = box[d];
-    g.dim[d] = dims[d];
-  }
-  g.inv = 1.0 / side;
-  k_nb_cells<<<(N + 127) / 128, 128, 0, st>>>(N, R, g, cell_of, cell_start, cell_cnt, items, rc2, start, cnt, tg,
-                                               sr, overflow);
+cudaError_t nb_pack(int N, const int* start, const int* cnt, const int* slots, int* tg, int* sr, cudaStream_t st) {
+  k_nb_pack<<<(int)(((long long)N * 8 + 127) / 128), 128, 0, st>>>(N, start, cnt, slots, tg, sr);
   return cudaGetLastError();
 }
 

@@ -23,7 +23,7 @@ constexpr int kSmallSystem = 4096;   // one system up to this size: O(N^2) neigh
 gbi_status build_pairs(gbi_ctx* ctx, int N, const double* R, double a, double rcut, int nsys,
                        const int* offsets_host, int& npair) {
   using namespace mlpk;
-  const double rc2 = (rcut * a) * (rcut * a);
+  const double rc = rcut * a, rc2 = rc * rc;
   const int* sys_of = nullptr;
   const int* sys_off = nullptr;
   Batch B;
@@ -34,48 +34,37 @@ gbi_status build_pairs(gbi_ctx* ctx, int N, const double* R, double a, double rc
   }
   GBI_TRY(ensure(ctx, ctx->nb_cnt, sizeof(int) * (size_t)N));
   GBI_TRY(ensure(ctx, ctx->nb_start, sizeof(int) * (size_t)(N + 1)));
-  GBI_TRY(ensure(ctx, ctx->nb_scan, sizeof(int) * scan_scratch_ints(N)));
-  GBI_TRY(ensure(ctx, ctx->nb_aux, 64 * 6 * sizeof(double) + 16));
+  GBI_TRY(ensure(ctx, ctx->nb_aux, 16));
   int* cnt = P<int>(ctx->nb_cnt);
   int* start = P<int>(ctx->nb_start);
   const bool cells = nsys <= 1 && N > kSmallSystem;
-  double box[6];
-  double side = rcut * a;
-  int dims[3] = {1, 1, 1};
-  int* overflow = reinterpret_cast<int*>(static_cast<char*>(ctx->nb_aux.p) + 64 * 6 * sizeof(double));
+  int* overflow = P<int>(ctx->nb_aux);
+  size_t scan_ints = scan_scratch_ints(N);
   if (cells) {
-    GBI_CHECK(mlpk::bbox(N, R, P<double>(ctx->nb_aux), box, ctx->stream));
-    double ext = 0.0;
-    for (int d = 0; d < 3; ++d) ext = std::max(ext, box[3 + d] - box[d]);
-    side = std::max(side, ext / 96.0);           // at most 97^3 cells
-    for (int d = 0; d < 3; ++d) dims[d] = std::max(1, (int)std::ceil((box[3 + d] - box[d]) / side));
-    const int nc = dims[0] * dims[1] * dims[2];
+    const int nc = 1 << nb_cell_bits(N);
     GBI_TRY(ensure(ctx, ctx->cell_of, sizeof(int) * (size_t)N));
+    GBI_TRY(ensure(ctx, ctx->cell_fill, sizeof(int) * (size_t)N));
     GBI_TRY(ensure(ctx, ctx->cell_cnt, sizeof(int) * (size_t)nc));
-    GBI_TRY(ensure(ctx, ctx->cell_start, sizeof(int) * (size_t)nc));
-    GBI_TRY(ensure(ctx, ctx->cell_fill, sizeof(int) * (size_t)nc));
-    GBI_TRY(ensure(ctx, ctx->cell_items, sizeof(int) * (size_t)N));
-    if (ensure(ctx, ctx->nb_scan, sizeof(int) * std::max(scan_scratch_ints(N), scan_scratch_ints(nc))) != GBI_OK)
-      return GBI_ERR_NOMEM;
-    GBI_CHECK(cells_build(N, R, box, side, dims, P<int>(ctx->cell_of), P<int>(ctx->cell_cnt),
-                          P<int>(ctx->cell_start), P<int>(ctx->cell_fill), P<int>(ctx->cell_items),
-                          P<int>(ctx->nb_scan), ctx->stream));
-    GBI_CHECK(cudaMemsetAsync(overflow, 0, sizeof(int), ctx->stream));
-    GBI_CHECK(nb_cells(N, R, box, side, dims, P<int>(ctx->cell_of), P<int>(ctx->cell_start), P<int>(ctx->cell_cnt),
-                       P<int>(ctx->cell_items), rc2, nullptr, cnt, nullptr, nullptr, overflow, ctx->stream));
-    ctx->launches += 6;
+    GBI_TRY(ensure(ctx, ctx->cell_start, sizeof(int) * (size_t)(nc + 1)));
+    GBI_TRY(ensure(ctx, ctx->cell_items, sizeof(float4) * (size_t)N));
+    GBI_TRY(ensure(ctx, ctx->nb_slots, sizeof(int) * nb_slot_ints(N)));
+    scan_ints = std::max(scan_ints, scan_scratch_ints(nc));
+  }
+  GBI_TRY(ensure(ctx, ctx->nb_scan, sizeof(int) * scan_ints));
+  if (cells) {
+    GBI_CHECK(nb_search(N, R, rc, rc2, P<int>(ctx->cell_of), P<int>(ctx->cell_fill), P<int>(ctx->cell_cnt),
+                        P<int>(ctx->cell_start), ctx->cell_items.p, P<int>(ctx->nb_scan), cnt, P<int>(ctx->nb_slots),
+                        overflow, ctx->stream));
+    ctx->launches += 4;
   } else {
-    GBI_CHECK(nb_count_sys(N, R, sys_of, sys_off, rc2, cnt, ctx->stream));
+    GBI_CHECK(nb_count_sys(N, R, sys_of, sys_off, nsys, rc, rc2, cnt, ctx->stream));
     ++ctx->launches;
   }
-  GBI_CHECK(exclusive_scan(cnt, start, N, P<int>(ctx->nb_scan), ctx->stream));
-  ctx->launches += 3;
-  const int chunks = (N + 1023) / 1024;
+  GBI_CHECK(exclusive_scan(cnt, start, N, start + N, P<int>(ctx->nb_scan), ctx->stream));
+  ++ctx->launches;
   int total = 0, ovf = 0;
-  GBI_CHECK(cudaMemcpyAsync(&total, P<int>(ctx->nb_scan) + chunks, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  GBI_CHECK(cudaMemcpyAsync(&total, start + N, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   if (cells) GBI_CHECK(cudaMemcpyAsync(&ovf, overflow, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  GBI_CHECK(cudaMemcpyAsync(start + N, P<int>(ctx->nb_scan) + chunks, sizeof(int), cudaMemcpyDeviceToDevice,
-                            ctx->stream));
   GBI_CHECK(cudaStreamSynchronize(ctx->stream));
   if (ovf) {
     ctx->err = "more than 64 neighbours within the cut-off for some sphere (overlapping input?)";
@@ -84,11 +73,10 @@ gbi_status build_pairs(gbi_ctx* ctx, int N, const double* R, double a, double rc
   GBI_TRY(ensure(ctx, ctx->nb_tg, sizeof(int) * (size_t)std::max(total, 1)));
   GBI_TRY(ensure(ctx, ctx->nb_sr, sizeof(int) * (size_t)std::max(total, 1)));
   if (cells)
-    GBI_CHECK(nb_cells(N, R, box, side, dims, P<int>(ctx->cell_of), P<int>(ctx->cell_start), P<int>(ctx->cell_cnt),
-                       P<int>(ctx->cell_items), rc2, start, nullptr, P<int>(ctx->nb_tg), P<int>(ctx->nb_sr), overflow,
-                       ctx->stream));
+    GBI_CHECK(nb_pack(N, start, cnt, P<int>(ctx->nb_slots), P<int>(ctx->nb_tg), P<int>(ctx->nb_sr), ctx->stream));
   else
-    GBI_CHECK(nb_fill_sys(N, R, sys_of, sys_off, rc2, start, P<int>(ctx->nb_tg), P<int>(ctx->nb_sr), ctx->stream));
+    GBI_CHECK(nb_fill_sys(N, R, sys_of, sys_off, nsys, rc, rc2, start, P<int>(ctx->nb_tg), P<int>(ctx->nb_sr),
+                          ctx->stream));
   ++ctx->launches;
   ctx->nb_pairs = total;
   ctx->nb_N = N;
