@@ -249,6 +249,67 @@ __device__ __forceinline__ void lab_grad_to_pair(int head, const float* fr, cons
   }
 }
 #endif
+// Ordered pairs k = (tg[k], sr[k]) of spheres with centres R and orientations p.
+struct PairInputs {
+  const double* R;
+  const double* p;
+  const int* tg;
+  const int* sr;
+  double a;
+};
+#ifdef __CUDACC__
+// Features f[9] and frame rows fr[9] (e_x, e_y, e_z) of pair k, FP32 after an FP64 difference
+// of the centres (definitions in gbi.h)
+__device__ __forceinline__ void pair_features(const PairInputs& in, int k, float* f, float* fr) {
+  const double* __restrict__ R = in.R;
+  const double* __restrict__ p = in.p;
+  const double a = in.a;
+  const int n = in.tg[k], m = in.sr[k];
+  const float rx = float(R[3 * (size_t)n] - R[3 * (size_t)m]);
+  const float ry = float(R[3 * (size_t)n + 1] - R[3 * (size_t)m + 1]);
+  const float rz = float(R[3 * (size_t)n + 2] - R[3 * (size_t)m + 2]);
+  const float pn[3] = {float(p[3 * (size_t)n]), float(p[3 * (size_t)n + 1]), float(p[3 * (size_t)n + 2])};
+  const float pm[3] = {float(p[3 * (size_t)m]), float(p[3 * (size_t)m + 1]), float(p[3 * (size_t)m + 2])};
+  const float r = sqrtf(rx * rx + ry * ry + rz * rz);
+  const float ez[3] = {rx / r, ry / r, rz / r};
+  float t[3];
+  float c = pn[0] * ez[0] + pn[1] * ez[1] + pn[2] * ez[2];
+  for (int i = 0; i < 3; ++i) t[i] = pn[i] - c * ez[i];
+  float t2 = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
+  if (t2 <= 1e-12f) {
+    c = pm[0] * ez[0] + pm[1] * ez[1] + pm[2] * ez[2];
+    for (int i = 0; i < 3; ++i) t[i] = pm[i] - c * ez[i];
+    t2 = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
+  }
+  if (t2 <= 1e-12f) {
+    int ax = 0;
+    if (fabsf(ez[1]) < fabsf(ez[0])) ax = 1;
+    if (fabsf(ez[2]) < fabsf(ax == 0 ? ez[0] : ez[1])) ax = 2;
+    const float eax = ax == 0 ? ez[0] : (ax == 1 ? ez[1] : ez[2]);
+    for (int i = 0; i < 3; ++i) t[i] = (i == ax ? 1.f : 0.f) - eax * ez[i];
+    t2 = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
+  }
+  const float inv = 1.0f / sqrtf(t2);
+  const float ex[3] = {t[0] * inv, t[1] * inv, t[2] * inv};
+  const float ey[3] = {ez[1] * ex[2] - ez[2] * ex[1], ez[2] * ex[0] - ez[0] * ex[2], ez[0] * ex[1] - ez[1] * ex[0]};
+  const float u = float(2.0 * a) / r;
+  const float d = fmaxf(r / float(a) - 2.0f, 0.01f);
+  f[0] = u;
+  f[1] = u * u * u;
+  f[2] = d;
+  f[3] = logf(d);
+  f[4] = pn[0] * ez[0] + pn[1] * ez[1] + pn[2] * ez[2];
+  f[5] = pn[0] * ex[0] + pn[1] * ex[1] + pn[2] * ex[2];
+  f[6] = pm[0] * ex[0] + pm[1] * ex[1] + pm[2] * ex[2];
+  f[7] = pm[0] * ey[0] + pm[1] * ey[1] + pm[2] * ey[2];
+  f[8] = pm[0] * ez[0] + pm[1] * ez[1] + pm[2] * ez[2];
+  for (int i = 0; i < 3; ++i) {
+    fr[i] = ex[i];
+    fr[3 + i] = ey[i];
+    fr[6 + i] = ez[i];
+  }
+}
+#endif
 size_t scan_scratch_ints(int n);
 cudaError_t exclusive_scan(const int* in, int* out, int n, int* total, int* scratch, cudaStream_t st);
 cudaError_t nb_count_sys(int N, const double* R, const int* sys_of, const int* sys_off, int nsys, double rc,
@@ -290,6 +351,9 @@ size_t packed_tc_bytes();
 cudaError_t pack_weights_tc(const float* theta, void* packed, cudaStream_t st);
 cudaError_t infer_tc(int P, const float* F, const float* FR, const void* packed, float* out, int* err, int num_sms,
                      int head, cudaStream_t st);
+// the same with the features of every pair formed in the kernel (lab-frame outputs)
+cudaError_t infer_tc_pairs(int P, const PairInputs& in, const void* packed, float* out, int* err, int num_sms, int head,
+                           cudaStream_t st);
 cudaError_t labels(int N, double s0, double sigma, const double* Vx, const double* Ox, const double* Vs,
                    const double* Os, double* out, double* sq_part, cudaStream_t st);
 // labels[n] = sigma / s0 * (QHx - QH1)[n][0..4], 0 (rows of h); block partial sums of squares

@@ -6,9 +6,8 @@
 // outputs, K = 16 per instruction) issued by a single thread, operands in shared
 // memory in the no-swizzle K-major core-matrix layout (8 rows x 16 bytes per core
 // matrix), the FP32 accumulator in tensor memory (128 lanes x 128 columns) read back
-// with tcgen05.ld by eight warps: a warp may only read the lane quarter of its warp
-// index mod 4, so warps w and w + 4 share lanes 32 (w mod 4) .. + 31 (pairs of the tile)
-// and each takes half of the 128 columns of the epilogue.  Completion of each MMA chain
+// with tcgen05.ld (a warp may only read the lane quarter of its warp index mod 4: one row,
+// a pair, per thread of a group of four warps).  Completion of each MMA chain
 // is signalled through an mbarrier (tcgen05.commit); every wait has an iteration limit
 // after which the kernel records an error, releases its tensor memory and returns.
 #include <cuda_bf16.h>
@@ -137,127 +136,176 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// the same load without its wait; the registers are defined only after tmem_ld_wait on them
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15}, [%16];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+// waits for the issued loads; names the registers so that no use of them moves ahead of it
+__device__ __forceinline__ void tmem_ld_wait(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 constexpr long long kWaitLimit = 1ll << 22;   // try_wait rounds before giving up
 
+// Inference tiles.  A block is kTcGroups groups of four warps that share the weights in shared
+// memory; each group takes its own 128-pair tiles with its own operand buffers, accumulator
+// (128 tensor-memory columns of the 512) and completion barrier, so that one group's MMA and
+// barrier latency hides behind the others' epilogues.  The hardware tanh bounds the kernel (384
+// per pair, 16 per clock and SM: 41 us for the 538 240 pairs of N = 10^5); measured with the
+// features formed in the kernel 87 us (ncu: XU pipe 51 % busy), against 94 us and a separate 45 us
+// feature pass with two blocks of eight warps per SM, one tile each.
+constexpr int kTcGroups = 4;
+constexpr int kTcThreads = kTcGroups * TM;
+
+struct TcGroup {
+  __nv_bfloat16 a1[TM * K1];       // layer-1 operand (features)
+  __nv_bfloat16 act[TM * NH];      // hidden-layer operand
+};
 struct TcSmem {
   __nv_bfloat16 w[PWEND];          // weights, core-matrix layout
   float bias[PBIAS];
-  __nv_bfloat16 a1[TM * K1];       // layer-1 operand (features)
-  __nv_bfloat16 act[TM * NH];      // hidden-layer operand
-  unsigned long long mbar;
+  TcGroup g[kTcGroups];
+  unsigned long long mbar[kTcGroups];
   uint32_t tmem_base;
-  int abort;
+  int abort[kTcGroups];
 };
+static_assert(sizeof(TcSmem) <= 227 * 1024, "one block per SM, within the shared-memory limit");
 
-constexpr int kTcThreads = 256;   // eight warps: two per tensor-memory lane quarter
-
-__global__ void __launch_bounds__(kTcThreads) k_infer_tc(int P, const float* __restrict__ F, const float* __restrict__ FR,
-                                                   const __nv_bfloat16* __restrict__ pk, float* __restrict__ out,
-                                                   int* __restrict__ err, int head) {
+// FUSED: the features and frames of pair k come from its spheres (in.tg[k], in.sr[k]) in the
+// kernel; otherwise from F and FR (FR null: pair-frame outputs)
+template <bool FUSED>
+__global__ void __launch_bounds__(kTcThreads, 1) k_infer_tc(int P, const float* __restrict__ F,
+                                                            const float* __restrict__ FR, const PairInputs in,
+                                                            const __nv_bfloat16* __restrict__ pk,
+                                                            float* __restrict__ out, int* __restrict__ err, int head) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   TcSmem& s = *reinterpret_cast<TcSmem*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int row = tid & (TM - 1);          // the pair of the tile (accumulator lane) this thread reads
-  const int half = warp >> 2;              // which 64 of the 128 hidden columns it handles
-  {
-    const int4* src = reinterpret_cast<const int4*>(pk);
-    int4* dst = reinterpret_cast<int4*>(s.w);
-    const int n16 = int((sizeof(__nv_bfloat16) * PWEND + sizeof(float) * PBIAS) / 16);
-    for (int i = tid; i < n16; i += blockDim.x) dst[i] = src[i];
-  }
-  const uint32_t mbar = saddr(&s.mbar);
-  if (tid == 0) {
-    s.abort = 0;
+  const int grp = tid / TM, row = tid & (TM - 1);   // row: the pair of the tile (accumulator lane)
+  const uint32_t mbar = saddr(&s.mbar[grp]);
+  if (row == 0) {
+    s.abort[grp] = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mbar), "r"(1) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(saddr(&s.tmem_base)),
-                 "r"(128)
+                 "r"(kTcGroups * NH)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  {
+    const int4* src = reinterpret_cast<const int4*>(pk);
+    int4* dst = reinterpret_cast<int4*>(s.w);
+    constexpr int n16 = int((sizeof(__nv_bfloat16) * PWEND + sizeof(float) * PBIAS) / 16);
+#pragma unroll 5
+    for (int i = tid; i < n16; i += kTcThreads) dst[i] = src[i];
   }
   fence_async_smem();
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = s.tmem_base;
+  const uint32_t tmem0 = s.tmem_base;
+  const uint32_t tmem = tmem0 + (uint32_t)(grp * NH);
   const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;   // this warp's TMEM lane quarter
-  const uint32_t a1_addr = saddr(s.a1), act_addr = saddr(s.act), w_addr = saddr(s.w);
+  TcGroup& sg = s.g[grp];
+  const uint32_t a1_addr = saddr(sg.a1), act_addr = saddr(sg.act), w_addr = saddr(s.w);
   const uint32_t id_hidden = instr_desc(TM, NH), id_out = instr_desc(TM, N4);
   uint32_t parity = 0;
   const int ntiles = (P + TM - 1) / TM;
+  auto group_sync = [&]() { asm volatile("bar.sync %0, %1;\n" ::"r"(grp + 1), "r"(TM) : "memory"); };
 
-  // issue one layer (thread 0) and wait for it (all threads); false if the wait gave up
+  // issue one layer (the group's first thread) and wait for it; false if the wait gave up
   auto run_layer = [&](uint32_t a_addr, int K, uint32_t b_addr, uint32_t idesc) -> bool {
     fence_async_smem();   // operands written through the generic proxy
     fence_before();
-    __syncthreads();
+    group_sync();
     fence_after();
-    if (tid == 0) {
-      const uint32_t sbo_a = (uint32_t)K * 16;   // 8 rows x K bf16
-      const uint32_t sbo_b = (uint32_t)K * 16;
-      for (int ks = 0; ks < K / 16; ++ks) {
-        const uint64_t ad = smem_desc(a_addr + ks * 256, 128, sbo_a);
-        const uint64_t bd = smem_desc(b_addr + ks * 256, 128, sbo_b);
-        mma_f16(tmem, ad, bd, idesc, ks > 0 ? 1u : 0u);
-      }
+    if (row == 0) {
+      const uint32_t sbo = (uint32_t)K * 16;   // 8 rows x K bf16
+      for (int ks = 0; ks < K / 16; ++ks)
+        mma_f16(tmem, smem_desc(a_addr + ks * 256, 128, sbo), smem_desc(b_addr + ks * 256, 128, sbo), idesc,
+                ks > 0 ? 1u : 0u);
       mma_commit(mbar);
     }
     long long it = 0;
     while (!mbar_try_wait(mbar, parity)) {
       if (++it > kWaitLimit) {
-        s.abort = 1;
+        s.abort[grp] = 1;
         break;
       }
     }
     parity ^= 1u;
     fence_after();
-    __syncthreads();
-    return s.abort == 0;
+    group_sync();
+    return s.abort[grp] == 0;
   };
 
-  // hidden epilogue: row `row`, columns [64 half, 64 half + 64) of the accumulator ->
-  // tanh(. + b) -> bf16 -> act (core layout)
+  // hidden epilogue: the thread's accumulator row -> tanh(. + b) -> bf16 -> act (core layout);
+  // the next 16 columns are on their way from tensor memory while these are evaluated
   auto hidden_epilogue = [&](const float* b) {
-#pragma unroll 1
-    for (int c0 = half * (NH / 2); c0 < (half + 1) * (NH / 2); c0 += 16) {
-      float v[16];
-      tmem_ld16(tmem + lane_base + (uint32_t)c0, v);
-      __align__(16) __nv_bfloat16 o[16];
+    uint32_t v[2][16];
+    tmem_ld16_issue(tmem + lane_base, v[0]);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) o[i] = __float2bfloat16_rn(tanh_act(v[i] + b[c0 + i]));
-      *reinterpret_cast<int4*>(&s.act[cm_index(row, c0, NH)]) = *reinterpret_cast<const int4*>(&o[0]);
-      *reinterpret_cast<int4*>(&s.act[cm_index(row, c0 + 8, NH)]) = *reinterpret_cast<const int4*>(&o[8]);
+    for (int c = 0; c < NH / 16; ++c) {
+      tmem_ld_wait(v[c & 1]);
+      if (c + 1 < NH / 16) tmem_ld16_issue(tmem + lane_base + (uint32_t)(16 * (c + 1)), v[(c + 1) & 1]);
+      __align__(16) __nv_bfloat162 o[8];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 bb = *reinterpret_cast<const float4*>(b + 16 * c + 4 * q);
+        const uint32_t* w = v[c & 1] + 4 * q;
+        o[2 * q] = __floats2bfloat162_rn(tanh_act(__uint_as_float(w[0]) + bb.x), tanh_act(__uint_as_float(w[1]) + bb.y));
+        o[2 * q + 1] = __floats2bfloat162_rn(tanh_act(__uint_as_float(w[2]) + bb.z), tanh_act(__uint_as_float(w[3]) + bb.w));
+      }
+      *reinterpret_cast<int4*>(&sg.act[cm_index(row, 16 * c, NH)]) = *reinterpret_cast<const int4*>(&o[0]);
+      *reinterpret_cast<int4*>(&sg.act[cm_index(row, 16 * c + 8, NH)]) = *reinterpret_cast<const int4*>(&o[4]);
     }
   };
 
   bool ok = true;
-  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+  // tiles go to the first groups of every block first, so that few tiles spread over the SMs
+  for (int tile = grp * gridDim.x + blockIdx.x; tile < ntiles; tile += kTcGroups * gridDim.x) {
     const int p = tile * TM + row;
-    if (half == 0) {
+    float fr[9];
+    {
+      float ft[NIN];
+#pragma unroll
+      for (int k = 0; k < NIN; ++k) ft[k] = 0.f;
+      if (p < P) {
+        if constexpr (FUSED) {
+          pair_features(in, p, ft, fr);
+        } else {
+#pragma unroll
+          for (int k = 0; k < NIN; ++k) ft[k] = F[(size_t)p * NIN + k];
+        }
+      }
       __align__(16) __nv_bfloat16 f[16];
 #pragma unroll
-      for (int k = 0; k < 16; ++k) f[k] = __float2bfloat16_rn((k < NIN && p < P) ? F[(size_t)p * NIN + k] : 0.f);
-      *reinterpret_cast<int4*>(&s.a1[cm_index(row, 0, K1)]) = *reinterpret_cast<const int4*>(&f[0]);
-      *reinterpret_cast<int4*>(&s.a1[cm_index(row, 8, K1)]) = *reinterpret_cast<const int4*>(&f[8]);
+      for (int k = 0; k < 16; ++k) f[k] = __float2bfloat16_rn(k < NIN ? ft[k < NIN ? k : 0] : 0.f);
+      *reinterpret_cast<int4*>(&sg.a1[cm_index(row, 0, K1)]) = *reinterpret_cast<const int4*>(&f[0]);
+      *reinterpret_cast<int4*>(&sg.a1[cm_index(row, 8, K1)]) = *reinterpret_cast<const int4*>(&f[8]);
     }
-    ok = run_layer(a1_addr, K1, w_addr + 2 * PW1, id_hidden);
-    if (!ok) break;
+    if (!(ok = run_layer(a1_addr, K1, w_addr + 2 * PW1, id_hidden))) break;
     hidden_epilogue(s.bias);
-    ok = run_layer(act_addr, NH, w_addr + 2 * PW2, id_hidden);
-    if (!ok) break;
+    if (!(ok = run_layer(act_addr, NH, w_addr + 2 * PW2, id_hidden))) break;
     hidden_epilogue(s.bias + NH);
-    ok = run_layer(act_addr, NH, w_addr + 2 * PW3, id_hidden);
-    if (!ok) break;
+    if (!(ok = run_layer(act_addr, NH, w_addr + 2 * PW3, id_hidden))) break;
     hidden_epilogue(s.bias + 2 * NH);
-    ok = run_layer(act_addr, NH, w_addr + 2 * PW4, id_out);
-    if (!ok) break;
-    if (half != 0) continue;   // the 16 output columns: the first warp of each lane quarter
+    if (!(ok = run_layer(act_addr, NH, w_addr + 2 * PW4, id_out))) break;
     float o[16];
     tmem_ld16(tmem + lane_base, o);
     if (p < P) {
@@ -266,7 +314,9 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(int P, const float* __r
 #pragma unroll
       for (int c = 0; c < NOUT; ++c) y[c] = o[c] + b4[c];
       float* dst = out + (size_t)p * NOUT;
-      if (FR != nullptr) {
+      if constexpr (FUSED) {
+        pair_out_to_lab(head, fr, y, dst);
+      } else if (FR != nullptr) {
         pair_out_to_lab(head, FR + (size_t)p * 9, y, dst);
       } else {
 #pragma unroll
@@ -280,11 +330,12 @@ __global__ void __launch_bounds__(kTcThreads) k_infer_tc(int P, const float* __r
     long long it = 0;
     while (!mbar_try_wait(mbar, parity ^ 1u) && ++it <= kWaitLimit) {
     }
-    if (tid == 0) atomicExch(err, 1);
+    if (row == 0) atomicExch(err, 1);
   }
   fence_before();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(128) : "memory");
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem0), "r"(kTcGroups * NH) : "memory");
 }
 
 // ---- training: backward pass on the tensor cores -------------------------------------
@@ -557,16 +608,28 @@ cudaError_t pack_weights_tc(const float* theta, void* packed, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t infer_tc(int P, const float* F, const float* FR, const void* packed, float* out, int* err, int num_sms,
-                     int head, cudaStream_t st) {
+template <bool FUSED>
+static cudaError_t launch_infer_tc(int P, const float* F, const float* FR, const PairInputs& in, const void* packed,
+                                   float* out, int* err, int num_sms, int head, cudaStream_t st) {
   if (P <= 0) return cudaSuccess;
   const size_t smem = sizeof(TcSmem);
-  cudaError_t e = cudaFuncSetAttribute(k_infer_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  cudaError_t e = cudaFuncSetAttribute(k_infer_tc<FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   const int ntiles = (P + TM - 1) / TM;
-  const int grid = ntiles < 2 * num_sms ? ntiles : 2 * num_sms;
-  k_infer_tc<<<grid, kTcThreads, smem, st>>>(P, F, FR, static_cast<const __nv_bfloat16*>(packed), out, err, head);
+  const int grid = ntiles < num_sms ? ntiles : num_sms;
+  k_infer_tc<FUSED><<<grid, kTcThreads, smem, st>>>(P, F, FR, in, static_cast<const __nv_bfloat16*>(packed), out, err,
+                                                    head);
   return cudaGetLastError();
+}
+
+cudaError_t infer_tc(int P, const float* F, const float* FR, const void* packed, float* out, int* err, int num_sms,
+                     int head, cudaStream_t st) {
+  return launch_infer_tc<false>(P, F, FR, PairInputs{}, packed, out, err, num_sms, head, st);
+}
+
+cudaError_t infer_tc_pairs(int P, const PairInputs& in, const void* packed, float* out, int* err, int num_sms, int head,
+                           cudaStream_t st) {
+  return launch_infer_tc<true>(P, nullptr, nullptr, in, packed, out, err, num_sms, head, st);
 }
 
 }  // namespace mlpk

@@ -106,7 +106,6 @@ gbi_status mlp_prepare(gbi_ctx* ctx, int N, const double* R, const double* p, do
   return GBI_OK;
 }
 
-
 // Network inference with the selected engine.  The tcgen05 kernel reports a wait that
 // gave up through a device flag that gbi_mlp_status reads back.
 gbi_status mlp_infer(gbi_ctx* ctx, int np_, const float* F, const float* FR, float* out) {
@@ -117,6 +116,23 @@ gbi_status mlp_infer(gbi_ctx* ctx, int np_, const float* F, const float* FR, flo
     return GBI_OK;
   }
   GBI_CHECK(mlpk::infer(np_, F, FR, ctx->mlp_pk.p, out, sm_count(ctx), ctx->mlp_head, ctx->stream));
+  ++ctx->launches;
+  return GBI_OK;
+}
+
+// The 4a pairs of R and their lab-frame outputs in ctx->mf_lab.  The tensor-core engine forms
+// the features in the inference kernel (72 bytes per pair neither written nor read back).
+gbi_status mlp_pair_outputs(gbi_ctx* ctx, int N, const double* R, const double* p, double a, int nsys,
+                            const int* offsets_host, int& npair) {
+  if (ctx->mlp_engine != 1) {
+    GBI_TRY(mlp_prepare(ctx, N, R, p, a, nsys, offsets_host, npair));
+    return mlp_infer(ctx, npair, P<float>(ctx->mf_F), P<float>(ctx->mf_FR), P<float>(ctx->mf_lab));
+  }
+  GBI_TRY(build_pairs(ctx, N, R, a, 4.0, nsys, offsets_host, npair));
+  GBI_TRY(ensure(ctx, ctx->mf_lab, sizeof(float) * 6 * (size_t)std::max(npair, 1)));
+  const mlpk::PairInputs in{R, p, P<int>(ctx->nb_tg), P<int>(ctx->nb_sr), a};
+  GBI_CHECK(mlpk::infer_tc_pairs(npair, in, ctx->mlp_pk_tc.p, P<float>(ctx->mf_lab), P<int>(ctx->mlp_err),
+                                 sm_count(ctx), ctx->mlp_head, ctx->stream));
   ++ctx->launches;
   return GBI_OK;
 }
@@ -247,8 +263,7 @@ gbi_status gbi_mlp_correct(gbi_ctx* ctx, int N, const double* R, const double* p
   if (N == 0) return GBI_OK;
   if (!R || !p || !V || !Omega) return GBI_ERR_ARG;
   int np_ = 0;
-  GBI_TRY(mlp_prepare(ctx, N, R, p, a, nsys, offsets_host, np_));
-  GBI_TRY(mlp_infer(ctx, np_, P<float>(ctx->mf_F), P<float>(ctx->mf_FR), P<float>(ctx->mf_lab)));
+  GBI_TRY(mlp_pair_outputs(ctx, N, R, p, a, nsys, offsets_host, np_));
   GBI_CHECK(mlpk::sphere_sums(N, P<int>(ctx->nb_start), P<float>(ctx->mf_lab), s0 / ctx->mlp_sigma, V, Omega,
                               ctx->stream));
   ctx->launches += 1;
@@ -269,8 +284,7 @@ gbi_status gbi_mlp_correct_qh(gbi_ctx* ctx, int N, const double* R, const double
   if (N == 0) return GBI_OK;
   if (!R || !p || !QH) return GBI_ERR_ARG;
   int np_ = 0;
-  GBI_TRY(mlp_prepare(ctx, N, R, p, a, nsys, offsets_host, np_));
-  GBI_TRY(mlp_infer(ctx, np_, P<float>(ctx->mf_F), P<float>(ctx->mf_FR), P<float>(ctx->mf_lab)));
+  GBI_TRY(mlp_pair_outputs(ctx, N, R, p, a, nsys, offsets_host, np_));
   GBI_CHECK(mlpk::sphere_sums_q(N, P<int>(ctx->nb_start), P<float>(ctx->mf_lab), s0 / ctx->mlp_sigma, QH, h,
                                 ctx->stream));
   ctx->launches += 1;
