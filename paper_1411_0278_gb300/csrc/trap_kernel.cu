@@ -426,12 +426,13 @@ static int trap_resident(int precision) {
 
 int trap_splits(int N, int precision) {
   // as many source splits as keep every target block's splits within one wave of the
-  // resident blocks (a wave and a few stragglers costs a second wave), at least 64
-  // sources per split
+  // resident blocks (a wave and a few stragglers costs a second wave), at least 64 sources
+  // per split (FP64: 16 -- a source costs 64 times the FP32 one, so filling the SMs pays for
+  // the extra partial sums earlier; at N = 1500 the 64-source splits were 69 blocks on 152 SMs)
   const int ti = trap_ti(precision);
   const int tblocks = (N + kThreads * ti - 1) / (kThreads * ti);
   int s = trap_resident(precision) / tblocks;
-  const int maxs = (N + 63) / 64;
+  const int maxs = precision == 1 ? (N + 63) / 64 : (N + 15) / 16;
   if (s > maxs) s = maxs;
   return s < 1 ? 1 : s;
 }

@@ -16,184 +16,106 @@
 //   8 pi eta u(x) = sum_m W_ij(x, R_m) F_j + D_jk d/dy_k W_ij(x, y)|_{y = R_m},
 //   D_jk = S_jk + (1/2) eps_kjl T_l,   V_n += u(R_n),   Omega_n += curl u (R_n) / 2.
 //
-// Derivatives are exact (to rounding): forward-mode dual numbers, nested.  The inner
-// level carries the three directional derivatives along the rows D_j. of the source's
-// dipole tensor (so its j-th component is D_jk d/dy_k), the outer one the derivatives
-// along the three axes at the target (for the curl).  One thread per target; sources in
-// shared-memory tiles; the sources are split over gridDim.y slices whose partial sums are
-// added in slice order by a second kernel, so the result does not depend on timing.
+// In closed form, with phi = 1/|R|, z = x_3 and m = (1, 1, -1): the bracket is
+// z d_i d_j phi - d_i3 d_j phi + d_j3 d_i phi, d/dy_k = -m_k d/dR_k (+ d/dh for k = 3), so with
+//   Dt_jk = -D_jk m_k,   E_j = m_j (h F_j + D_j3),   H_jk = h m_j Dt_jk (symmetrised),   c_k = h m_3 Dt_3k,
+//   Phi = -E.R/|R|^3 + 3 (R.H R)/|R|^5 - tr H / |R|^3,   chi = E_3/|R| - (c.R)/|R|^3
+// (both harmonic), and q = R.Dt R, v = Dt R, a_i = eps_ijk Dt_jk,
+//   u = -F/|R| - (F.R) R/|R|^3 - (a x R + tr Dt R)/|R|^3 + 3 q R/|R|^5 + 2 (z grad Phi - e_3 Phi + grad chi),
+//   curl u = -2 (F x R + a)/|R|^3 + 6 (v x R)/|R|^5 + 4 e_3 x grad Phi.
+// Everything that depends on the source alone is formed once per source (k_wall_records), so a
+// pair costs about 100 floating-point instructions (nested dual numbers, which this replaces:
+// 1 089 in the compiled FP32 kernel).  Measured, with the unbounded superposition: FP64 N = 1500
+// 5.73 -> 1.02 ms, FP32 N = 10^4 4.29 -> 0.85 ms; the error against 64 bits of the FP32 sums fell from
+// 2.9e-7 to 1.9e-7 (N = 4000), that of the FP64 sums is 1e-15.
+// Sources in shared-memory tiles, split over gridDim.y slices whose partial sums are added in
+// slice order by a second kernel, so the result does not depend on timing.
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <type_traits>
 
 #include "ctx.cuh"
+#include "df.cuh"
 #include "gbi_generated.cuh"
 
 namespace gbi {
 namespace {
 
 constexpr int kWallThreads = 128;
-constexpr int kWallTile = 64;
-constexpr int kWallRec = 16;   // per source: x y z, F (3), D (9, row-major), pad
+constexpr int kWallTile = 32;
+constexpr int kWallRec = 32;   // words per source record (layout at k_wall_records)
 
-// Flops of one (target, source) term (FMA = 2) as the compiled FP32 kernel executes them:
-// 392.6 FFMA and 696 other FP32 instructions per term (ncu instruction statistics of the
-// N = 10^4 launch).  The nested dual numbers as written would count 4 096 -- a D2 product
-// is 82 flops -- but most derivative entries are structurally zero (the target-side
-// derivatives of the source height, the constant derivatives of R) and fold away.
-constexpr int kWallPairFlops = 1481;
-
-// ---------------------------------------------------------------------------------
-// dual numbers: a value and its derivatives along three directions.  D1 = Dual3<T>
-// (inner, source side), D2 = Dual3<D1> (outer, target side).
-// ---------------------------------------------------------------------------------
-template <typename U> struct Dual3 {
-  U v;
-  U d[3];
-};
-
-template <typename U> __device__ __forceinline__ Dual3<U> operator+(const Dual3<U>& a, const Dual3<U>& b) {
-  Dual3<U> r;
-  r.v = a.v + b.v;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r.d[k] = a.d[k] + b.d[k];
-  return r;
-}
-template <typename U> __device__ __forceinline__ Dual3<U> operator-(const Dual3<U>& a, const Dual3<U>& b) {
-  Dual3<U> r;
-  r.v = a.v - b.v;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r.d[k] = a.d[k] - b.d[k];
-  return r;
-}
-template <typename U> __device__ __forceinline__ Dual3<U> operator*(const Dual3<U>& a, const Dual3<U>& b) {
-  Dual3<U> r;
-  r.v = a.v * b.v;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r.d[k] = a.v * b.d[k] + a.d[k] * b.v;
-  return r;
-}
-// scaling by a plain number
-template <typename U, typename T, typename = typename std::enable_if<std::is_arithmetic<T>::value>::type>
-__device__ __forceinline__ Dual3<U> operator*(T s, const Dual3<U>& a) {
-  Dual3<U> r;
-  r.v = s * a.v;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r.d[k] = s * a.d[k];
-  return r;
-}
+// Flops of one (target, source) term as written below (FMA = 2, rsqrt = 1)
+constexpr int kWallPairFlops = 170;
 
 __device__ __forceinline__ float wall_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double wall_rsqrt(double x) { return rsqrt(x); }
 
-// a^(-1/2) and its derivatives: (a^-1/2)' = -1/2 a^-3/2
-template <typename T> __device__ __forceinline__ Dual3<T> rsqrt1(const Dual3<T>& a) {
-  Dual3<T> r;
-  r.v = wall_rsqrt(a.v);
-  const T f1 = T(-0.5) * r.v * r.v * r.v;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r.d[k] = f1 * a.d[k];
-  return r;
-}
-template <typename T> __device__ __forceinline__ Dual3<Dual3<T>> rsqrt2(const Dual3<Dual3<T>>& a) {
-  Dual3<Dual3<T>> r;
-  r.v = rsqrt1(a.v);
-  const Dual3<T> f1 = T(-0.5) * (r.v * r.v * r.v);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r.d[k] = f1 * a.d[k];
-  return r;
-}
-
-template <typename T> __device__ __forceinline__ Dual3<T> d1_const(T v) {
-  Dual3<T> r;
-  r.v = v;
-  r.d[0] = r.d[1] = r.d[2] = T(0);
-  return r;
-}
-template <typename T> __device__ __forceinline__ Dual3<Dual3<T>> d2_const(T v) {
-  Dual3<Dual3<T>> r;
-  r.v = d1_const(v);
-  r.d[0] = r.d[1] = r.d[2] = d1_const(T(0));
-  return r;
-}
-
-// Image flow at target x (times 8 pi eta) of a source at y with force F and dipole D:
-// u_i += W_ij F_j + D_jk dW_ij/dy_k, and the derivatives du_i/dx_l into the curl c.
+// a x b + c
 template <typename T>
-__device__ __forceinline__ void wall_image_pair(const T* x, const T* src, T* u, T* c) {
-  using D1 = Dual3<T>;
-  using D2 = Dual3<D1>;
-  const T* y = src;
-  const T* F = src + 3;
-  const T* D = src + 6;   // D[3 j + k] = D_jk
-  // R_k = x_k - y*_k: outer derivative d/dx_l = delta_kl, inner (direction j) derivative
-  // D_jk dR_k/dy_k = -D_jk (k = 0, 1) or +D_j2 (k = 2: R_3 = x_3 + y_3)
-  D2 R[3];
+__device__ __forceinline__ void cross_add(const T* a, const T* b, T c0, T c1, T c2, T* o) {
+  o[0] = gbi_fmac(a[1], b[2], gbi_fmac(-a[2], b[1], c0));
+  o[1] = gbi_fmac(a[2], b[0], gbi_fmac(-a[0], b[2], c1));
+  o[2] = gbi_fmac(a[0], b[1], gbi_fmac(-a[1], b[0], c2));
+}
+
+// Image flow at target x (times 8 pi eta) of the source record r added to u, its curl to c.
+template <typename T>
+__device__ __forceinline__ void wall_image_pair(const T* x, const T* __restrict__ r, T* u, T* c) {
+  const T R[3] = {x[0] - r[0], x[1] - r[1], x[2] + r[2]};
+  const T* F = r + 3;     // F
+  const T* Dt = r + 6;    // Dt, row-major
+  const T* a = r + 15;    // a
+  const T* H = r + 18;    // 2 H: xx xy xz yy yz zz
+  const T* E = r + 24;    // 2 E
+  const T* cc = r + 27;   // 2 c
+  const T tr = r[30];     // tr Dt + 2 E_3
+  const T th = r[31];     // 2 tr H
+  const T r2 = gbi_fmac(R[2], R[2], gbi_fmac(R[1], R[1], R[0] * R[0]));
+  const T i1 = wall_rsqrt(r2);
+  const T i2 = i1 * i1, i3 = i1 * i2, i5 = i3 * i2;
+  const T FR = gbi_fmac(F[2], R[2], gbi_fmac(F[1], R[1], gbi_fmac(F[0], R[0], tr)));
+  const T v[3] = {gbi_fmac(Dt[2], R[2], gbi_fmac(Dt[1], R[1], Dt[0] * R[0])),
+                  gbi_fmac(Dt[5], R[2], gbi_fmac(Dt[4], R[1], Dt[3] * R[0])),
+                  gbi_fmac(Dt[8], R[2], gbi_fmac(Dt[7], R[1], Dt[6] * R[0]))};
+  const T q = gbi_fmac(R[2], v[2] + cc[2], gbi_fmac(R[1], v[1] + cc[1], R[0] * (v[0] + cc[0])));
+  const T g[3] = {gbi_fmac(H[2], R[2], gbi_fmac(H[1], R[1], H[0] * R[0])),
+                  gbi_fmac(H[4], R[2], gbi_fmac(H[3], R[1], H[1] * R[0])),
+                  gbi_fmac(H[5], R[2], gbi_fmac(H[4], R[1], H[2] * R[0]))};
+  const T qh = gbi_fmac(R[2], g[2], gbi_fmac(R[1], g[1], R[0] * g[0]));
+  const T ER = gbi_fmac(E[2], R[2], gbi_fmac(E[1], R[1], gbi_fmac(E[0], R[0], th)));
+  // 2 Phi and 2 grad Phi = 6 g i5 - E i3 + kp R
+  const T t5 = T(3) * i5;
+  const T phi = gbi_fmac(t5, qh, -(ER * i3));
+  const T kp = gbi_fmac(T(-15) * i2, qh, T(3) * ER) * i5;
+  const T s5 = T(6) * i5;
+  T dp[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) dp[k] = gbi_fmac(s5, g[k], gbi_fmac(-i3, E[k], kp * R[k]));
+  // u: the R-parallel terms of the Oseen part and grad chi, the others, z 2 grad Phi - 2 e_3 Phi;
+  // a pair's terms are added together before the sum takes them (one rounding against the sum:
+  // accumulating term by term measured 20 % more FP32 error)
+  const T k0 = gbi_fmac(t5, q, -(FR * i3));
+  T w[3];
+  cross_add<T>(a, R, cc[0], cc[1], cc[2], w);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const T sgn = k == 2 ? T(1) : T(-1);
-    R[k].v.v = k == 2 ? x[2] + y[2] : x[k] - y[k];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) R[k].v.d[j] = sgn * D[3 * j + k];
-#pragma unroll
-    for (int l = 0; l < 3; ++l) R[k].d[l] = d1_const(l == k ? T(1) : T(0));
+    const T pre = k == 2 ? -gbi_fmac(i1, F[k], phi) : -(i1 * F[k]);
+    u[k] += gbi_fmac(x[2], dp[k], gbi_fmac(k0, R[k], gbi_fmac(-i3, w[k], pre)));
   }
-  // h = y_3: inner derivative D_j2, no outer derivative
-  D2 h = d2_const(y[2]);
-#pragma unroll
-  for (int j = 0; j < 3; ++j) h.v.d[j] = D[3 * j + 2];
-  // shared factors (D2 products: 6 + 3 + 1 + 1 + 3 = 14; sums and scalings: 2 + 1 + 1)
-  D2 RR[6];                                         // R_i R_j, i <= j
-  RR[0] = R[0] * R[0];
-  RR[1] = R[0] * R[1];
-  RR[2] = R[0] * R[2];
-  RR[3] = R[1] * R[1];
-  RR[4] = R[1] * R[2];
-  RR[5] = R[2] * R[2];
-  const D2 iR = rsqrt2(RR[0] + RR[3] + RR[5]);
-  const D2 iR2 = iR * iR;
-  const D2 iR3 = iR2 * iR;
-  const D2 iR5 = iR3 * iR2;
-  const D2 hR3 = h * iR3;
-  const D2 c5 = T(3) * ((R[2] - h) * iR5);          // 3 (R_3 - h) / |R|^5
-  D2 RiR3[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) RiR3[k] = R[k] * iR3;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int lo = i < j ? i : j, hi = i < j ? j : i;
-      const D2& Rij = RR[lo == 0 ? hi : (lo == 1 ? 2 + hi : 5)];
-      // Oseen tensor at R, and the bracket of the image terms (per entry: 3 D2 products,
-      // up to 4 sums and 1 scaling)
-      D2 g = Rij * iR3;
-      D2 t = Rij * c5;
-      if (i == j) {
-        g = g + iR;
-        t = t + hR3 - RiR3[2];
-      }
-      if (i == 2) t = t + RiR3[j];
-      if (j == 2) t = t - RiR3[i];
-      const D2 w = T(2 * (j == 2 ? -1 : 1)) * (h * t) - g;
-      u[i] += w.v.v * F[j] + w.v.d[j];
-      // du_i/dx_l = w.d[l].v F_j + w.d[l].d[j]; curl c = (d2u3 - d3u2, d3u1 - d1u3, d1u2 - d2u1)
-#pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        const T dl = w.d[l].v * F[j] + w.d[l].d[j];
-        if (i == 2 && l == 1) c[0] += dl;
-        if (i == 1 && l == 2) c[0] -= dl;
-        if (i == 0 && l == 2) c[1] += dl;
-        if (i == 2 && l == 0) c[1] -= dl;
-        if (i == 1 && l == 0) c[2] += dl;
-        if (i == 0 && l == 1) c[2] -= dl;
-      }
-    }
-  }
+  // curl: -2 (F x R + a) i3 + 6 (v x R) i5 + 2 e_3 x (2 grad Phi)
+  T f[3], vr[3];
+  cross_add<T>(F, R, a[0], a[1], a[2], f);
+  cross_add<T>(v, R, T(0), T(0), T(0), vr);
+  const T m3 = T(-2) * i3;
+  c[0] += gbi_fmac(T(-2), dp[1], gbi_fmac(m3, f[0], s5 * vr[0]));
+  c[1] += gbi_fmac(T(2), dp[0], gbi_fmac(m3, f[1], s5 * vr[1]));
+  c[2] += gbi_fmac(m3, f[2], s5 * vr[2]);
 }
 
-// Source records: position, force, dipole D = S + A(T) in T.
+// Source records: 0..2 position, 3..5 F, 6..14 Dt, 15..17 a, 18..23 2 H, 24..26 2 E, 27..29 2 c,
+// 30 tr Dt + 2 E_3, 31 2 tr H -- formed in FP64 and rounded to T.
 template <typename T>
 __global__ void k_wall_records(int N, double a, double eta, const double* __restrict__ R,
                                const double* __restrict__ VH, int h, const double* __restrict__ Fe,
@@ -206,21 +128,45 @@ __global__ void k_wall_records(int N, double a, double eta, const double* __rest
   gbi_unpack2<double>(VH + (size_t)h * m, s6);
   const double S[9] = {s6[0], s6[1], s6[2], s6[1], s6[3], s6[4], s6[2], s6[4], s6[5]};
   const double T0 = Te[3 * (size_t)m], T1 = Te[3 * (size_t)m + 1], T2 = Te[3 * (size_t)m + 2];
-  // A_jk = (1/2) eps_kjl T_l
+  // D = S + A, A_jk = (1/2) eps_kjl T_l
   const double A[9] = {0.0, -0.5 * T2, 0.5 * T1, 0.5 * T2, 0.0, -0.5 * T0, -0.5 * T1, 0.5 * T0, 0.0};
+  const double sg[3] = {1.0, 1.0, -1.0};
+  const double y3 = R[3 * (size_t)m + 2];
+  double F[3], D[9], Dt[9], E[3], Hf[9];
+  for (int k = 0; k < 3; ++k) F[k] = Fe[3 * (size_t)m + k];
+  for (int q = 0; q < 9; ++q) D[q] = cs * S[q] + A[q];
+  for (int j = 0; j < 3; ++j) {
+    for (int k = 0; k < 3; ++k) {
+      Dt[3 * j + k] = -sg[k] * D[3 * j + k];
+      Hf[3 * j + k] = y3 * sg[j] * Dt[3 * j + k];
+    }
+    E[j] = sg[j] * (y3 * F[j] + D[3 * j + 2]);
+  }
   for (int k = 0; k < 3; ++k) {
     o[k] = T(R[3 * (size_t)m + k]);
-    o[3 + k] = T(Fe[3 * (size_t)m + k]);
+    o[3 + k] = T(F[k]);
+    o[24 + k] = T(2.0 * E[k]);
+    o[27 + k] = T(2.0 * Hf[6 + k]);
   }
-  for (int q = 0; q < 9; ++q) o[6 + q] = T(cs * S[q] + A[q]);
-  o[15] = T(0);
+  for (int q = 0; q < 9; ++q) o[6 + q] = T(Dt[q]);
+  o[15] = T(Dt[5] - Dt[7]);
+  o[16] = T(Dt[6] - Dt[2]);
+  o[17] = T(Dt[1] - Dt[3]);
+  o[18] = T(2.0 * Hf[0]);
+  o[19] = T(Hf[1] + Hf[3]);
+  o[20] = T(Hf[2] + Hf[6]);
+  o[21] = T(2.0 * Hf[4]);
+  o[22] = T(Hf[5] + Hf[7]);
+  o[23] = T(2.0 * Hf[8]);
+  o[30] = T(Dt[0] + Dt[4] + Dt[8] + 2.0 * E[2]);
+  o[31] = T(2.0 * (Hf[0] + Hf[4] + Hf[8]));
 }
 
 // Partial image sums of the targets over the sources of slice blockIdx.y.
 template <typename T>
 __global__ void __launch_bounds__(kWallThreads) k_wall_pairs(int N, int per_slice, const T* __restrict__ rec,
                                                              T* __restrict__ part) {
-  __shared__ T s_rec[kWallTile * kWallRec];
+  __shared__ __align__(32) T s_rec[kWallTile * kWallRec];
   const int n = blockIdx.x * kWallThreads + threadIdx.x;
   const int m0 = blockIdx.y * per_slice;
   const int m1 = min(N, m0 + per_slice);
@@ -246,25 +192,34 @@ __global__ void __launch_bounds__(kWallThreads) k_wall_pairs(int N, int per_slic
 }
 
 // V += u / (8 pi eta), Omega += c / (16 pi eta), the slices added in order.
+// One thread per (sphere, component), component fastest, eight slices' loads in flight.
 template <typename T>
 __global__ void k_wall_reduce(int N, int slices, double eta, const T* __restrict__ part, double* V, double* Om) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  double s[6] = {0, 0, 0, 0, 0, 0};
-  for (int q = 0; q < slices; ++q)
-    for (int k = 0; k < 6; ++k) s[k] += double(part[((size_t)q * N + n) * 6 + k]);
-  const double f = 1.0 / (8.0 * kPi * eta);
-  for (int k = 0; k < 3; ++k) {
-    V[3 * (size_t)n + k] += f * s[k];
-    Om[3 * (size_t)n + k] += 0.5 * f * s[3 + k];
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long rows = 6LL * N;
+  if (i >= rows) return;
+  const long long n = i / 6;
+  const int c = (int)(i - 6 * n);
+  double acc = 0.0;
+  for (int q = 0; q < slices; q += 8) {
+    T p[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) p[k] = q + k < slices ? part[(long long)(q + k) * rows + i] : T(0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (q + k < slices) acc += double(p[k]);
   }
+  const double f = 1.0 / (8.0 * kPi * eta);
+  if (c < 3) V[3 * n + c] += f * acc;
+  else Om[3 * n + c - 3] += 0.5 * f * acc;
 }
 
 int wall_slices(int N) {
-  // about four blocks per SM on 152 SMs, at least 32 sources per slice
+  // about four blocks per SM on 152 SMs, at least 8 sources per slice: at small N the slices
+  // are the only parallelism, and a source costs a thread a chain of dependent operations
   const int tb = (N + kWallThreads - 1) / kWallThreads;
   int s = (608 + tb - 1) / tb;
-  const int maxs = (N + 31) / 32;
+  const int maxs = (N + 7) / 8;
   if (s > maxs) s = maxs;
   return s < 1 ? 1 : s;
 }
@@ -278,7 +233,7 @@ cudaError_t launch_wall_t(int N, double a, double eta, const double* R, const do
   T* part = rec + (size_t)N * kWallRec;
   k_wall_records<T><<<(N + 255) / 256, 256, 0, st>>>(N, a, eta, R, VH, h, Fe, Te, rec);
   k_wall_pairs<T><<<dim3((N + kWallThreads - 1) / kWallThreads, slices), kWallThreads, 0, st>>>(N, per, rec, part);
-  k_wall_reduce<T><<<(N + 255) / 256, 256, 0, st>>>(N, slices, eta, part, V, Om);
+  k_wall_reduce<T><<<(unsigned)((6LL * N + 127) / 128), 128, 0, st>>>(N, slices, eta, part, V, Om);
   return cudaGetLastError();
 }
 
