@@ -294,6 +294,7 @@ cudaError_t run_pairs(gbi_ctx* ctx, int trunc, int rows, int cols, int precision
     args.wpt = ctx->force_wpt > 0 ? ctx->force_wpt
                                   : ctx->tuned_wpt(trunc, rows, cols, precision, args.N,
                                                    args.sys_of != nullptr && args.nsys > 1);
+  if (precision == 0 || ctx->force_wpt > 0) args.group = 0;
   tile_select(ctx, trunc, rows, precision, args);
   if (precision >= 1 && !balanced_form(args.wpt) && !(args.sys_of != nullptr && args.nsys > 1) &&
       ctx->split_tail)
@@ -500,6 +501,8 @@ PairArgs pair_args(const Setup& s, const double* x, double* y, double alpha, dou
   p.wait_limit = 0;
   p.split_from = 0x7fffffff;
   p.nsplit = 1;
+  p.group = 0;
+  p.y_sphere = 0;
   return p;
 }
 
@@ -536,6 +539,7 @@ gbi_status single_batch(gbi_ctx* ctx, int N, Batch& B) {
   B.one[0] = 0;
   B.one[1] = N;
   B.h_off = B.one;
+  B.max_n = N;
   return GBI_OK;
 }
 
@@ -576,7 +580,22 @@ gbi_status make_batch(gbi_ctx* ctx, int nsys, const int* offsets_host, Batch& B)
   B.off = P<int>(ctx->boff);
   B.sys = P<int>(ctx->bsys);
   B.h_off = offsets_host;
+  B.max_n = 0;
+  for (int q = 0; q < nsys; ++q) B.max_n = std::max(B.max_n, offsets_host[q + 1] - offsets_host[q]);
   return GBI_OK;
+}
+
+// The group form serves batches whose every system has at most 33 spheres: a warp then holds
+// all the sources of a target at once, where the other forms give it two warps or more.  The
+// streaming form stays for larger systems (its lanes fill) and where a warps-per-target choice
+// is forced.
+constexpr int kGroupMaxSystem = 33;
+
+int group_lanes(const Batch& B) {
+  if (B.S <= 1 || B.max_n > kGroupMaxSystem) return 0;
+  int g = 1;
+  while (g < B.max_n - 1) g <<= 1;
+  return g;
 }
 
 bool valid_params(const gbi_params* p) {

@@ -50,7 +50,7 @@ struct gbi_ctx {
   bool fixed = false;                            // buffers bound to static storage: never reallocate
   cudaGraphExec_t chunk_exec = nullptr;          // device-looped Arnoldi steps of one GMRES cycle
   const void* chunk_key[8] = {};                 // buffers and sizes the graph was built for
-  long long chunk_ikey[6] = {};
+  long long chunk_ikey[8] = {};
   int chunk_nodes = 0;                           // kernels per loop iteration
   // the whole mixed-precision solve as one graph: built when a call repeats the previous
   // call's key (buffers, sizes, parameters, tuning), replayed while the key stays
@@ -232,6 +232,7 @@ struct Batch {
   const int* sys = nullptr;   // device [Ntot]
   const int* h_off = nullptr; // host copy of off (the caller's array, or one[] below)
   int one[2] = {0, 0};        // offsets of the single-system case
+  int max_n = 0;              // spheres of the largest system
   Batch() = default;
   Batch(const Batch&) = delete;   // h_off may point into the object
   Batch& operator=(const Batch&) = delete;
@@ -240,6 +241,8 @@ struct Batch {
 bool valid_params(const gbi_params* p);
 // ordered pairs of a batch, sum over its systems of n (n - 1)
 long long batch_pairs(const Batch& B);
+// lanes per target of the group form for a batch, 0 where the other forms serve it
+int group_lanes(const Batch& B);
 bool valid_offsets(int nsys, const int* off);
 gbi_status make_batch(gbi_ctx* ctx, int nsys, const int* offsets_host, Batch& B);
 gbi_status single_batch(gbi_ctx* ctx, int N, Batch& B);

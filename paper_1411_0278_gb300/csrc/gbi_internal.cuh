@@ -80,6 +80,9 @@ struct PairArgs {
   // tile_part (doubles, 32-row chunks) and the last to arrive (tile_cnt, one counter per
   // split target, zero between launches) adds the parts in part order and stores
   int split_from, nsplit;
+  // batches of small systems: lanes that share a target (pair_group_kernel), 0 for the other forms
+  int group;
+  int y_sphere;          // group form: y is [N][rows] instead of component-major
 };
 
 // Programmatic dependent launch: with pdl set the kernel's blocks may be scheduled while

@@ -463,7 +463,7 @@ __device__ __forceinline__ void stream_source(const PairArgs& args, const float4
 
 // Row p (counted from the pass's first row) of target n in the streaming forms: the
 // pair sum (units 1/a), the self term, then y = alpha v + beta y.
-template <int TR, int ROWS, int COLS, typename T>
+template <int TR, int ROWS, int COLS, typename T, bool SPHERE = false>
 __device__ __forceinline__ void store_target(const PairArgs& args, int n, int p, double sum) {
   using S = PassShape<TR, ROWS, COLS>;
   constexpr int R0 = S::R0;
@@ -481,7 +481,7 @@ __device__ __forceinline__ void store_target(const PairArgs& args, int n, int p,
                          : double(args.x32[(size_t)n * (RECV * 4) + q]);
     v += args.selfg[R0 + p] * inva * xs;
   }
-  double* dst = args.y + (size_t)p * args.N + n;
+  double* dst = args.y + (SPHERE && args.y_sphere ? (size_t)n * S::NR + p : (size_t)p * args.N + n);
   *dst = args.alpha * v + (args.beta != 0.0 ? args.beta * (*dst) : 0.0);
 }
 
@@ -581,6 +581,78 @@ __global__ void __launch_bounds__(WPT * 32, MINB) pair_stream_kernel(const PairA
     const int p = 32 * c + lane;
     if (p < NR) store_target<TR, ROWS, COLS, T>(args, n, p, gbi_to_double(tot[c]));
   }
+}
+
+// ---------------------------------------------------------------------------------
+// Group form for batches of small systems (PairArgs::group).
+//
+// A sphere of a system of n has n - 1 sources, so with a block of warps per target nearly
+// every lane idles when the systems are small.  Here `group` lanes (a power of two up to 32,
+// at least n - 1 of the largest system where that is possible) share a target: lane j takes
+// the sources j, j + group, ... of the n - 1 others, so 32 / group targets share a warp, and a
+// butterfly over the group's lanes adds the partial sums (fixed order).  4000 systems of two
+// and three spheres at l <= 4 (ncu): H/H 14 us in FP32 and 81 us in double-float, against 86 and 758 us
+// with two warps per target.  The rows are split over the lanes before they are stored: the
+// stores' FP64 scaling (16 cycles a warp instruction) costs as much as the pairs.
+// ---------------------------------------------------------------------------------
+template <int TR, int ROWS, int COLS, typename T, int THREADS, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB) pair_group_kernel(const PairArgs args) {
+  using S = PassShape<TR, ROWS, COLS>;
+  constexpr int NR = S::NR;
+  pdl_wait();
+  if (args.active != nullptr && *args.active == 0) return;   // device-side GMRES has stopped
+  const int G = args.group;
+  const int t = (blockIdx.x * THREADS + threadIdx.x) / G;
+  const int sub = threadIdx.x & (G - 1);
+  const int n = min(t, args.N - 1);
+  const int sy = args.sys_of[n];
+  const bool live =
+      t < args.N && (args.sys_flag == nullptr || args.sys_flag[(size_t)sy * args.sys_flag_stride] != 0);
+  const int lo = args.sys_off[sy], others = args.sys_off[sy + 1] - lo - 1;
+  const T a = T(args.a);
+  const float4 th = args.pos.hi[n], tl = args.pos.lo[n];
+  const float4* __restrict__ rec = reinterpret_cast<const float4*>(args.x32);
+  T acc[NR];
+#pragma unroll
+  for (int p = 0; p < NR; ++p) acc[p] = T(0);
+  float min_r2 = 3.0e38f;
+  if (live)
+    for (int j = sub; j < others; j += G) {
+      const int m = lo + j + (lo + j >= n ? 1 : 0);
+      stream_source<TR, ROWS, COLS, T>(args, rec, th, tl, m, a, acc, min_r2);
+    }
+  // lanes of the group: the first exchange halves the rows (even lanes keep the first half, odd
+  // lanes the second), the others add them up
+  constexpr int NH = (NR + 1) / 2;
+  const bool odd = (sub & 1) != 0;
+  if (G > 1) {
+#pragma unroll
+    for (int p = 0; p < NH; ++p) {
+      const T up = p + NH < NR ? acc[p + NH < NR ? p + NH : p] : T(0);
+      const T keep = odd ? up : acc[p], send = odd ? acc[p] : up;
+      acc[p] = keep + gbi_shfl(send, 1);
+    }
+    for (int o = 2; o < G; o <<= 1) {
+#pragma unroll
+      for (int p = 0; p < NH; ++p) acc[p] = acc[p] + gbi_shfl(acc[p], o);
+    }
+  }
+  if (args.min_r2_bits != nullptr) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) min_r2 = fminf(min_r2, __shfl_xor_sync(0xffffffffu, min_r2, o));
+    if ((threadIdx.x & 31) == 0) atomicMin(args.min_r2_bits, __float_as_uint(min_r2));
+  }
+  if (!live) return;
+  if (G == 1) {
+#pragma unroll
+    for (int p = 0; p < NR; ++p) store_target<TR, ROWS, COLS, T, true>(args, n, p, gbi_to_double(acc[p]));
+    return;
+  }
+  const int base = odd ? NH : 0, half = G >> 1;
+#pragma unroll
+  for (int p = 0; p < NH; ++p)
+    if ((p & (half - 1)) == (sub >> 1) && base + p < NR)
+      store_target<TR, ROWS, COLS, T, true>(args, n, base + p, gbi_to_double(acc[p]));
 }
 
 }  // namespace gbi

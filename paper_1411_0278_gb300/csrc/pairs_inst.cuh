@@ -77,6 +77,21 @@ cudaError_t launch_pairs_tt(int rows, int cols, const PairArgs& args, cudaStream
 #undef GBI_T
       return cudaErrorInvalidValue;
     }
+    if (args.group > 0) {
+      // lanes-per-target form of small systems: blocks of 64 (8 resident warps) or 128 threads
+      constexpr int THREADS = WARPS_SM >= 16 ? 128 : 64;
+      const int per = THREADS / args.group;
+#define GBI_G(RV, CV)                                                                              \
+  if (rows == RV && cols == CV) {                                                                  \
+    return launch_pdl(args.pdl != 0, dim3((N + per - 1) / per), dim3(THREADS), stream,             \
+                      pair_group_kernel<TRN, RV, CV, T, THREADS, WARPS_SM * 32 / THREADS>, args);  \
+  }
+      GBI_G(SET_H, SET_L)
+      GBI_G(SET_H, SET_H)
+      GBI_G(SET_L, SET_ALL)
+#undef GBI_G
+      return cudaErrorInvalidValue;
+    }
     const int wpt = stream_wpt(TRN, DF ? 2 : 1, N, args.wpt);
 #define GBI_S(RV, CV, WPT)                                                                         \
   if (rows == RV && cols == CV && wpt == WPT) {                                                    \

@@ -661,6 +661,180 @@ __global__ void __launch_bounds__(256) bk_step_fused(double* V, size_t n, double
   }
 }
 
+// The whole orthogonalisation of the one-reduction step for batches of small systems
+// (warp_systems): one warp per system, kStepWarps systems per block, against one block per
+// system for the dot products and the Givens step and a second kernel for the vectors.  GB300's
+// FP64 pipe (a warp instruction takes 16 cycles of the SM's, whatever its active lanes) bounds it,
+// so the FP64 instructions are what is saved: a lane's elements of w stay in registers (only the
+// groups of 32 that the system fills are touched); four slots are reduced together by halving
+// (6 additions instead of 20); and the serial part -- |w - sum c_i V_i|^2 = |w|^2 - sum c_i^2, the
+// rotations, the stopping test -- runs for all systems of the block at once, one lane each.  The
+// last block to finish (counted in cnt[S]) ends the step as loop_continue does.  4000 systems of
+// two and three spheres, l <= 4: 31 us a step (ncu, 64 % of the FP64 pipe at the seventh step; 39 us
+// with the serial part on one lane of every warp and full shuffle trees).
+// In this form w and the basis are sphere-major ([Ntot][h]: a system's vector is contiguous, so a
+// warp's loads touch two cache lines instead of one per component row), the basis vector V_i in
+// slot i + 1 of the Krylov buffer (slot 0 holds the component-major residual the cycle started
+// from).
+constexpr int kWarpElems = 256;
+constexpr int kStepWarps = 4;
+
+__global__ void __launch_bounds__(32 * kStepWarps) bk_step_warp(double* __restrict__ Vb, size_t n,
+                                                                const double* __restrict__ w, int Ntot, int h,
+                                                                const int* __restrict__ off, GPtr p, SrcOut so,
+                                                                LoopCtl lc) {
+  pdl_wait();
+  extern __shared__ double s_step[];   // per system: col[m + 2], cs[m], sn[m]
+  __shared__ double s_ihn[kStepWarps];
+  __shared__ int s_go[kStepWarps];
+  const int m = p.m, stride = 3 * m + 2;
+  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int s = blockIdx.x * kStepWarps + wi;
+  const bool act = s < p.S && p.st[s].active != 0;
+  const int j = act ? p.st[s].j : 0;
+  double* col = s_step + wi * stride;
+  const int lo = act ? off[s] : 0, len = act ? (off[s + 1] - lo) * h : 0;
+  const int kmax = (len + 31) >> 5;
+  // element e = lane + 32 k of the system; lanes past its end read element 0 and hold w = 0
+  const size_t t0 = (size_t)lo * h;
+  double* V = Vb + n + t0;
+  double wr[kWarpElems / 32];
+  int ix[kWarpElems / 32];
+#pragma unroll
+  for (int k = 0; k < kWarpElems / 32; ++k) {
+    const int e = lane + 32 * k;
+    ix[k] = e < len ? e : 0;
+    wr[k] = e < len ? w[t0 + e] : 0.0;
+  }
+  if (act) {
+    const size_t o1 = (size_t)s * (m + 1);
+    for (int i = lane; i < j; i += 32) {
+      col[m + 2 + i] = p.cs[o1 + i];
+      col[2 * m + 2 + i] = p.sn[o1 + i];
+    }
+    // slots 0..j: V_i . w; slot j + 1: w . w
+    for (int i0 = 0; i0 <= j + 1; i0 += 4) {
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u;
+        if (i <= j) {
+          const double* v = V + (size_t)i * n;
+#pragma unroll
+          for (int k = 0; k < kWarpElems / 32; ++k)
+            if (k < kmax) a[u] = fma(v[ix[k]], wr[k], a[u]);
+        } else if (i == j + 1) {
+#pragma unroll
+          for (int k = 0; k < kWarpElems / 32; ++k)
+            if (k < kmax) a[u] = fma(wr[k], wr[k], a[u]);
+        }
+      }
+      const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
+      double b0 = (u16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, u16 ? a[0] : a[2], 16);
+      const double b1 = (u16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, u16 ? a[1] : a[3], 16);
+      b0 = (u8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, u8 ? b0 : b1, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) b0 += __shfl_xor_sync(0xffffffffu, b0, o);
+      const int i = i0 + (lane >> 3);   // lanes 0, 8, 16, 24 hold slots i0 .. i0 + 3
+      if ((lane & 7) == 0 && i <= j + 1) col[i] = b0;
+    }
+    __syncwarp();
+    // w - sum c_i V_i, before the rotations overwrite the coefficients
+    for (int i = 0; i <= j; ++i) {
+      const double c = col[i];
+      const double* v = V + (size_t)i * n;
+#pragma unroll
+      for (int k = 0; k < kWarpElems / 32; ++k)
+        if (k < kmax) wr[k] = fma(-c, v[ix[k]], wr[k]);
+    }
+  }
+  __syncthreads();
+  if (wi == 0 && lane < kStepWarps) {
+    // lane: one system of the block (inactive ones pass through)
+    const int q = blockIdx.x * kStepWarps + lane;
+    s_go[lane] = 0;
+    if (q < p.S && p.st[q].active) {
+      GDev* st = p.st + q;
+      const size_t o1 = (size_t)q * (m + 1);
+      double* c = s_step + lane * stride;
+      const double *cs = c + m + 2, *sn = cs + m;
+      const int jq = st->j;
+      const double gj = p.g[o1 + jq], ibn = st->inv_bnorm, tol = st->tol;
+      const int iters = st->iters + 1, maxit = st->max_iter;
+      double nrm = c[jq + 1];
+      for (int i = 0; i <= jq; ++i) nrm = fma(-c[i], c[i], nrm);
+      double hn, ihn;
+      root_and_inverse(nrm, hn, ihn);
+      double carry = c[0];
+      for (int i = 0; i < jq; ++i) {
+        const double t2 = c[i + 1], ci = cs[i], si = sn[i];
+        c[i] = ci * carry + si * t2;
+        carry = -si * carry + ci * t2;
+      }
+      double den, inv;
+      root_and_inverse(carry * carry + hn * hn, den, inv);
+      const double cc = den > 0 ? carry * inv : 1.0, sg = den > 0 ? hn * inv : 0.0;
+      c[jq] = den;
+      c[jq + 1] = 0.0;
+      const double g1 = -sg * gj;
+      const double res = fabs(g1) * ibn;
+      const int conv = res <= tol, brk = hn <= 1e-300;
+      const bool stop = conv || brk || iters >= maxit || jq + 1 >= m;
+      p.cs[o1 + jq] = cc;
+      p.sn[o1 + jq] = sg;
+      p.g[o1 + jq + 1] = g1;
+      p.g[o1 + jq] = cc * gj;
+      st->iters = iters;
+      st->kdim = jq + 1;
+      st->res = res;
+      st->converged = conv;
+      st->breakdown = brk;
+      if (stop) {
+        st->active = 0;
+      } else {
+        st->inv_hn = ihn;
+        st->j = jq + 1;
+        s_ihn[lane] = ihn;
+        s_go[lane] = 1;
+        atomicAdd(p.nact, 1);
+      }
+    }
+  }
+  __syncthreads();
+  if (act) {
+    double* H = p.H + (size_t)s * (m + 1) * m;
+    for (int i = lane; i <= j + 1; i += 32) H[(size_t)i * m + j] = col[i];
+    if (s_go[wi]) {
+      const double ihn = s_ihn[wi];
+#pragma unroll
+      for (int k = 0; k < kWarpElems / 32; ++k) {
+        const int e = lane + 32 * k;
+        if (e < len) {
+          const double v = wr[k] * ihn;
+          V[(size_t)(j + 1) * n + e] = v;
+          const int r = e / h;
+          write_src(so, Ntot, h, e - r * h, lo + r, v);
+        }
+      }
+    }
+  }
+  if (!lc.on) return;
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(p.cnt + p.S, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last || threadIdx.x != 0) return;
+  __threadfence();
+  p.cnt[p.S] = 0u;
+  const int v = *static_cast<volatile int*>(lc.nact);
+  *lc.nact = 0;
+  if (lc.on == 2) {
+    if (lc.steps != nullptr) *lc.steps += 1;
+    cudaGraphSetConditional(lc.h, v > 0 ? 1u : 0u);
+  }
+}
+
 // start of a GMRES cycle for system s (enabled systems): beta = |V_0|, g = (beta, 0, ...);
 // `first` marks the first cycle of an inner solve (the counters restart)
 __device__ void init_cycle_sys(const GPtr& p, int s, int first) {
@@ -704,6 +878,19 @@ __global__ void bk_scale0(double* V0, int Ntot, const int* __restrict__ sys, con
   const double v = V0[t] * g.inv_hn;
   V0[t] = v;
   write_src(src, Ntot, gridDim.y, blockIdx.y, p, v);
+}
+
+// bk_scale0 into the sphere-major basis of bk_step_warp: V_0 = residual / beta in slot 1
+__global__ void bk_scale0_warp(double* __restrict__ Vb, size_t n, int Ntot, int h, const int* __restrict__ sys,
+                               const GDev* __restrict__ st, SrcOut src) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int p = int(t / h), q = int(t - (size_t)p * h);
+  const GDev& g = st[sys[p]];
+  if (!g.active) return;
+  const double v = Vb[(size_t)q * Ntot + p] * g.inv_hn;
+  Vb[n + t] = v;
+  write_src(src, Ntot, h, q, p, v);
 }
 
 // End of a GMRES cycle in the solve graph, once every system's cycle is over: count the
@@ -822,6 +1009,23 @@ __global__ void bk_update(const double* __restrict__ V, size_t n, int Ntot, cons
   u[t] += minv.v[blockIdx.y] * acc;
 }
 
+// bk_update from the sphere-major basis of bk_step_warp
+__global__ void bk_update_warp(const double* __restrict__ Vb, size_t n, int Ntot, int h, const int* __restrict__ sys,
+                               GPtr p, Scales minv, double* u) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int pp = int(t / h), q = int(t - (size_t)pp * h);
+  const int s = sys[pp];
+  const int k = p.st[s].kdim;
+  if (k == 0) return;
+  const double* y = p.y + (size_t)s * (p.m + 1);
+  const double* V = Vb + n + t;
+  double acc = 0.0;
+#pragma unroll 4
+  for (int i = 0; i < k; ++i) acc += y[i] * V[(size_t)i * n];
+  u[(size_t)q * Ntot + pp] += minv.v[q] * acc;
+}
+
 // refinement bookkeeping of system s: mode 0 stores |b_s| (from nrm), mode 1 sets rel and
 // enabled, mode 2 sets rel only (the FP32 residual of a warm start's guess, which sizes
 // the first inner solve but decides nothing: only the high-precision residual may stop a
@@ -858,6 +1062,41 @@ struct NormCtl {
   int max_refine, max_iter;
   int incr;                          // kFollowSweep: residuals after the first sweep are updates
 };
+
+__device__ __forceinline__ void norm_follow(const GPtr& p, int s, const NormCtl& nc) {
+  switch (nc.follow) {
+    case kFollowCycle: init_cycle_sys(p, s, nc.d != nullptr ? nc.d->first : nc.first); break;
+    case kFollowRefine0: refine_sys(p, s, 0, nc.rtol); break;
+    case kFollowRefine1:
+    case kFollowSweep: refine_sys(p, s, 1, nc.rtol); break;
+    case kFollowWarm: refine_sys(p, s, 2, nc.rtol); break;
+    default: break;
+  }
+}
+
+// the sweep decision of the solve graph, by the block that finds every system's refinement
+// flag final
+__device__ __forceinline__ void sweep_decision(const GPtr& p, const NormCtl& nc) {
+  __threadfence();
+  int any = 0;
+  for (int q = threadIdx.x; q < p.S; q += blockDim.x) any |= __ldcg(&p.st[q].enabled);
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) {
+    p.cnt[p.S] = 0u;
+    DSolve* d = nc.d;
+    // the residual just tested: the high-precision pass (the first sweep, or every sweep
+    // without updates) or the FP32 update r -= A_32 d of the previous sweep's inner solve
+    if (nc.incr && d->refinements > 0)
+      d->mv32 += 1;
+    else
+      d->mv64 += 1;
+    d->refinements += 1;
+    const int go = any && d->refinements < nc.max_refine && d->iters < nc.max_iter;
+    d->ifs += go;
+    cudaGraphSetConditional(nc.hif, go ? 1u : 0u);
+    cudaGraphSetConditional(nc.hsw, go ? 1u : 0u);
+  }
+}
 
 // |x_s|^2 per system (partials per row chunk as bk_norm_part forms them, added by one warp
 // in a fixed order), followed in the same kernel by what uses it: every block (s, c) counts
@@ -904,14 +1143,7 @@ __global__ void __launch_bounds__(256) bk_norm_then(const double* __restrict__ x
   }
   if (threadIdx.x == 0) {
     p.cnt[s] = 0u;
-    switch (nc.follow) {
-      case kFollowCycle: init_cycle_sys(p, s, nc.d != nullptr ? nc.d->first : nc.first); break;
-      case kFollowRefine0: refine_sys(p, s, 0, nc.rtol); break;
-      case kFollowRefine1:
-      case kFollowSweep: refine_sys(p, s, 1, nc.rtol); break;
-      case kFollowWarm: refine_sys(p, s, 2, nc.rtol); break;
-      default: break;
-    }
+    norm_follow(p, s, nc);
     s_glob = 0;
     if (nc.follow == kFollowSweep) {
       if (enabled0) atomicAdd(reinterpret_cast<unsigned long long*>(&nc.d->pairs), (unsigned long long)sys_pairs(off, s));
@@ -921,26 +1153,50 @@ __global__ void __launch_bounds__(256) bk_norm_then(const double* __restrict__ x
   }
   __syncthreads();
   if (!s_glob) return;
-  // the sweep decision, once every system's refinement flag is final
-  __threadfence();
-  int any = 0;
-  for (int q = threadIdx.x; q < p.S; q += blockDim.x) any |= __ldcg(&p.st[q].enabled);
-  any = __syncthreads_or(any);
-  if (threadIdx.x == 0) {
-    p.cnt[p.S] = 0u;
-    DSolve* d = nc.d;
-    // the residual just tested: the high-precision pass (the first sweep, or every sweep
-    // without updates) or the FP32 update r -= A_32 d of the previous sweep's inner solve
-    if (nc.incr && d->refinements > 0)
-      d->mv32 += 1;
-    else
-      d->mv64 += 1;
-    d->refinements += 1;
-    const int go = any && d->refinements < nc.max_refine && d->iters < nc.max_iter;
-    d->ifs += go;
-    cudaGraphSetConditional(nc.hif, go ? 1u : 0u);
-    cudaGraphSetConditional(nc.hsw, go ? 1u : 0u);
+  sweep_decision(p, nc);
+}
+
+// bk_norm_then for batches of small systems (warp_systems): one warp per system sums its
+// vector (lanes stride the elements, a shuffle tree adds them) and lane 0 runs the follow-up;
+// four systems per block.  4000 systems of two and three spheres, l <= 4: 9.6 us against
+// 99 us with a 256-thread block and its nine barriers per system.
+__global__ void __launch_bounds__(128) bk_norm_warp(const double* __restrict__ x, int Ntot, int h,
+                                                    const int* __restrict__ off, GPtr p, int mode, NormCtl nc) {
+  if (nc.follow == kFollowCycle && blockIdx.x == 0 && threadIdx.x == 0) {
+    *p.nact = 0;
+    if (nc.d != nullptr) cudaGraphSetConditional(nc.ha, 1u);
   }
+  const int s = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (s < p.S) {
+    const GDev* st = p.st + s;
+    const bool want = norm_wanted(*st, mode);
+    const int enabled0 = st->enabled;
+    __syncwarp();   // every lane has read the state that lane 0 may change below
+    if (want) {
+      const int lo = off[s], ns = off[s + 1] - lo, len = ns * h;
+      double acc = 0.0;
+      for (int e = lane; e < len; e += 32) {
+        const int q = e / ns;
+        const double v = x[(size_t)q * Ntot + lo + (e - q * ns)];
+        acc += v * v;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) p.nrm[s] = acc;
+    }
+    if (lane == 0) {
+      norm_follow(p, s, nc);
+      if (nc.follow == kFollowSweep && enabled0)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&nc.d->pairs), (unsigned long long)sys_pairs(off, s));
+    }
+  }
+  if (nc.follow != kFollowSweep) return;
+  __shared__ int s_glob;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_glob = atomicAdd(p.cnt + p.S, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (s_glob) sweep_decision(p, nc);
 }
 
 // x += d on enabled systems
@@ -973,14 +1229,24 @@ SrcOut src_out(const Setup& s, int precision, void* xsrc) {
   return o;
 }
 
-// Largest system of a batch (spheres), and the vector length up to which the one-round
-// step gives each system a single block (bk_dots_sys)
-int max_system(const Batch& B) {
-  int mx = 0;
-  for (int q = 0; q < B.S; ++q) mx = std::max(mx, B.h_off[q + 1] - B.h_off[q]);
-  return mx;
-}
+// Vector length of the largest system up to which the one-round step gives each system a
+// single block (bk_dots_sys)
 constexpr long long kSysBlockElems = 4096;
+// ... and up to which a warp runs a system's whole step, norms included (bk_step_warp,
+// bk_norm_warp): eight elements per lane.  Used for batches of at least 64 systems, whose pair
+// passes then run in the group form (no warps-per-target choice forced).
+bool warp_systems(const gbi_ctx* ctx, const Batch& B, int h) {
+  return B.S >= 64 && (long long)B.max_n * h <= kWarpElems && ctx->force_wpt == 0 && group_lanes(B) > 0;
+}
+
+// |x_s|^2 and what follows it (bk_norm_then), a warp per system where the systems are tiny
+void launch_norm(gbi_ctx* ctx, const Batch& B, int h, const GPtr& gp, const double* x, int mode, const NormCtl& nc) {
+  if (warp_systems(ctx, B, h))
+    bk_norm_warp<<<(B.S + 3) / 4, 128, 0, ctx->stream>>>(x, B.Ntot, h, B.off, gp, mode, nc);
+  else
+    bk_norm_then<<<dim3(B.S, gp.CH), 256, 0, ctx->stream>>>(x, B.Ntot, h, B.off, gp, mode, nc);
+  ++ctx->launches;
+}
 
 // Gram-Schmidt of the Arnoldi step.  The FP64 solve (precision 0) orthogonalises twice
 // (CGS2) and takes the norm of the result.  The FP32 inner solves of the refinement
@@ -995,6 +1261,26 @@ int two_pass_gs(int precision) { return precision == 0 ? 1 : 0; }
 // node overhead on GB300 besides its kernels, a step after its system has stopped about
 // 4 us (its kernels return at once), so several steps a trip pay off.
 constexpr int kArnoldiUnroll = 4;
+
+// V_0 and its source at the start of a cycle, the solution update at its end
+void launch_scale0(gbi_ctx* ctx, const Setup& s, const Batch& B, const GPtr& gp, double* Vb, const SrcOut& so,
+                   int precision) {
+  const size_t n = (size_t)B.Ntot * s.h;
+  if (!two_pass_gs(precision) && warp_systems(ctx, B, s.h))
+    bk_scale0_warp<<<grid1(n), 256, 0, ctx->stream>>>(Vb, n, B.Ntot, s.h, B.sys, gp.st, so);
+  else
+    bk_scale0<<<dim3((B.Ntot + 255) / 256, s.h), 256, 0, ctx->stream>>>(Vb, B.Ntot, B.sys, gp.st, so);
+  ++ctx->launches;
+}
+void launch_update(gbi_ctx* ctx, const Setup& s, const Batch& B, const GPtr& gp, const double* Vb, double* u,
+                   int precision) {
+  const size_t n = (size_t)B.Ntot * s.h;
+  if (!two_pass_gs(precision) && warp_systems(ctx, B, s.h))
+    bk_update_warp<<<grid1(n), 256, 0, ctx->stream>>>(Vb, n, B.Ntot, s.h, B.sys, gp, s.minv, u);
+  else
+    bk_update<<<dim3((B.Ntot + 255) / 256, s.h), 256, 0, ctx->stream>>>(Vb, n, B.Ntot, B.sys, gp, s.minv, u);
+  ++ctx->launches;
+}
 
 // kChunk Arnoldi iterations of every active system: pair pass on the source of V_j
 // (written by the previous bk_scale / bk_scale0 / bk_sub_scale), classical Gram-Schmidt
@@ -1016,11 +1302,13 @@ gbi_status launch_chunk(gbi_ctx* ctx, const Setup& s, const Batch& B, int precis
   pa.nsys = B.S;
   pa.npairs = batch_pairs(B);
   pa.sys_off = B.off;
+  pa.group = group_lanes(B);
   pa.sys_flag = &gp.st[0].active;
   pa.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
   const SrcOut so = src_out(s, precision, xsrc);
   const dim3 gd(S, m + 1, gp.CH);
   const int two = two_pass_gs(precision);
+  pa.y_sphere = !two && warp_systems(ctx, B, h) ? 1 : 0;
   // programmatic dependent launch inside the one-reduction step, between kernels of the
   // same sequence (the first pair pass of a chunk follows other work)
   const bool pdl = ctx->pdl && !two;
@@ -1057,12 +1345,18 @@ gbi_status launch_chunk(gbi_ctx* ctx, const Setup& s, const Batch& B, int precis
       bk_finalize<<<S, 128, 0, ctx->stream>>>(gp, 1);
       bk_scale<<<g2, 256, 0, ctx->stream>>>(Vb, n, w, Ntot, B.sys, gp.st, so, lcs);
       ctx->launches += 7;
+    } else if (warp_systems(ctx, B, h)) {
+      // many tiny systems: a warp runs the rest of a system's step
+      GBI_CHECK(launch_pdl_smem(pdl, dim3((S + kStepWarps - 1) / kStepWarps), dim3(32 * kStepWarps),
+                                sizeof(double) * kStepWarps * (3 * m + 2), ctx->stream, bk_step_warp, Vb, n, w, Ntot,
+                                h, B.off, gp, so, lcs));
+      ++ctx->launches;
     } else {
       if (S < 64) {
         // dot products, norm and Givens step in one kernel
         GBI_CHECK(launch_pdl(pdl, gd, dim3(256), ctx->stream, bk_dots_fin, Vb, n, w, Ntot, h, B.off, gp));
         ++ctx->launches;
-      } else if ((long long)max_system(B) * h <= kSysBlockElems) {
+      } else if ((long long)B.max_n * h <= kSysBlockElems) {
         // many small systems: one block each
         bk_dots_sys<<<S, 256, 0, ctx->stream>>>(Vb, n, w, Ntot, h, B.off, gp);
         ++ctx->launches;
@@ -1139,10 +1433,10 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
   const bool graphs = ctx->allow_graphs && ctx->stream != nullptr && !ctx->prof;
   if (graphs) {
     const void* key[8] = {Vb, w, xsrc, ctx->gstate.p, B.sys, B.off, s.pos.hi, s.pos.p64};
-    const long long ikey[6] = {(long long)n, S, m, precision, s.trunc, Ntot};
+    const long long ikey[8] = {(long long)n, S, m, precision, s.trunc, Ntot, B.max_n, ctx->wpt_gen};
     bool same = ctx->chunk_exec != nullptr;
     for (int i = 0; i < 8 && same; ++i) same = ctx->chunk_key[i] == key[i];
-    for (int i = 0; i < 6 && same; ++i) same = ctx->chunk_ikey[i] == ikey[i];
+    for (int i = 0; i < 8 && same; ++i) same = ctx->chunk_ikey[i] == ikey[i];
     if (!same) {
       if (ctx->chunk_exec) cudaGraphExecDestroy(ctx->chunk_exec);
       ctx->chunk_exec = nullptr;
@@ -1176,7 +1470,7 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
       if (st != GBI_OK) return st;
       GBI_CHECK(e);
       for (int i = 0; i < 8; ++i) ctx->chunk_key[i] = key[i];
-      for (int i = 0; i < 6; ++i) ctx->chunk_ikey[i] = ikey[i];
+      for (int i = 0; i < 8; ++i) ctx->chunk_ikey[i] = ikey[i];
     }
   }
   bool first = true;
@@ -1190,6 +1484,7 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
       pr.nsys = B.S;
       pr.npairs = batch_pairs(B);
       pr.sys_off = B.off;
+      pr.group = group_lanes(B);
       pr.sys_flag = &gp.st[0].enabled;
       pr.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
       GBI_CHECK(run_pairs(ctx, s.trunc, SET_H, SET_H, precision, pr));
@@ -1203,10 +1498,9 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
       NormCtl nc{};
       nc.follow = kFollowCycle;
       nc.first = first ? 1 : 0;
-      bk_norm_then<<<dim3(S, gp.CH), 256, 0, ctx->stream>>>(Vb, Ntot, h, B.off, gp, 1, nc);
+      launch_norm(ctx, B, h, gp, Vb, 1, nc);
     }
-    bk_scale0<<<g2, 256, 0, ctx->stream>>>(Vb, Ntot, B.sys, gp.st, src_out(s, precision, xsrc));
-    ctx->launches += 2;
+    launch_scale0(ctx, s, B, gp, Vb, src_out(s, precision, xsrc), precision);
     GBI_CHECK(cudaGetLastError());
     if (first)
       for (int q = 0; q < S; ++q) before[q] = 0;      // the first cycle restarts the counters
@@ -1259,8 +1553,8 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
       }
     }
     bk_solve_y<<<S, 128, 0, ctx->stream>>>(gp);
-    bk_update<<<g2, 256, 0, ctx->stream>>>(Vb, n, Ntot, B.sys, gp, s.minv, u);
-    ctx->launches += 2;
+    ++ctx->launches;
+    launch_update(ctx, s, B, gp, Vb, u, precision);
     GBI_CHECK(cudaGetLastError());
     bool restart_any = false;
     for (int q = 0; q < S; ++q) {
@@ -1454,6 +1748,7 @@ gbi_status emit_gmres(GraphBuild& gb, const Setup& s, const Batch& B, const GPtr
     pr.nsys = B.S;
     pr.npairs = batch_pairs(B);
     pr.sys_off = B.off;
+    pr.group = group_lanes(B);
     pr.sys_flag = &gp.st[0].enabled;
     pr.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
     pr.active = &d->notfirst;   // u is zero in the first cycle
@@ -1464,16 +1759,15 @@ gbi_status emit_gmres(GraphBuild& gb, const Setup& s, const Batch& B, const GPtr
       nc.follow = kFollowCycle;
       nc.d = d;
       nc.ha = ha;
-      bk_norm_then<<<dim3(S, gp.CH), 256, 0, ctx->stream>>>(Vb, Ntot, h, B.off, gp, 1, nc);
+      launch_norm(ctx, B, h, gp, Vb, 1, nc);
     }
-    bk_scale0<<<g2, 256, 0, ctx->stream>>>(Vb, Ntot, B.sys, gp.st, src_out(s, 1, xsrc));
-    ctx->launches += 2;
+    launch_scale0(ctx, s, B, gp, Vb, src_out(s, 1, xsrc), 1);
     GBI_TRY(gb.body(gb.node(ha, cudaGraphCondTypeWhile), kBodyStep, [&]() -> gbi_status {
       return launch_chunk(ctx, s, B, 1, gp, m, Vb, w, xsrc, kArnoldiUnroll, false, LoopCtl{gp.nact, ha, 1, &d->steps});
     }));
     bk_solve_y<<<S, 128, 0, ctx->stream>>>(gp, d, B.off, hr);
-    bk_update<<<g2, 256, 0, ctx->stream>>>(Vb, n, Ntot, B.sys, gp, s.minv, u);
-    ctx->launches += 2;
+    ++ctx->launches;
+    launch_update(ctx, s, B, gp, Vb, u, 1);
     GBI_CHECK(cudaGetLastError());
     return GBI_OK;
   }));
@@ -1529,6 +1823,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
     p.nsys = B.S;
     p.npairs = batch_pairs(B);
     p.sys_off = B.off;
+    p.group = group_lanes(B);
     p.sys_flag = flag;
     p.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
     return p;
@@ -1620,7 +1915,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
     }
     const void* ptrs[] = {B.sys, B.off, ctx->pos_hi.p, ctx->pos_lo.p, ctx->pos64.p, ctx->xQ.p, ctx->b.p, ctx->r.p, ctx->delta.p, ctx->xVL.p, ctx->minr2.p,
                           ctx->krylov.p, ctx->w.p, ctx->x32.p, ctx->gstate.p, ctx->dsolve.p, ctx->tile.p, ctx->tilecnt.p};
-    std::vector<long long> key = {N, S, pairs_all, max_system(B), prm->trunc, prm->precision, restart, max_iter,
+    std::vector<long long> key = {N, S, pairs_all, B.max_n, prm->trunc, prm->precision, restart, max_iter,
                                   max_refine,
                                   bits(rtol), bits(inner), bits(prm->min_sep), bits(prm->a), bits(prm->eta),
                                   ctx->wpt_gen, ctx->force_wpt, warm ? 1 : 0};
@@ -1664,8 +1959,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
                 NormCtl nc{};
                 nc.follow = kFollowRefine0;
                 nc.rtol = rtol;
-                bk_norm_then<<<dim3(S, gp.CH), 256, 0, ctx->stream>>>(b, N, h, B.off, gp, 2, nc);
-                ++ctx->launches;
+                launch_norm(ctx, B, h, gp, b, 2, nc);
               }
               gk_guard<<<1, 256, 0, ctx->stream>>>(gp, P<unsigned int>(ctx->minr2), bad_in, s.a,
                                                    pairs_all > 0 ? prm->min_sep : 0.0, d);
@@ -1687,8 +1981,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
                 NormCtl nc{};
                 nc.follow = kFollowWarm;
                 nc.rtol = rtol;
-                bk_norm_then<<<dim3(S, gp.CH), 256, 0, ctx->stream>>>(r, N, h, B.off, gp, 1, nc);
-                ++ctx->launches;
+                launch_norm(ctx, B, h, gp, r, 1, nc);
                 GBI_CHECK(cudaMemsetAsync(dl, 0, sizeof(double) * nh, ctx->stream));
                 GBI_TRY(emit_gmres(gb, s, B, gp, restart, r, dl, inner, max_iter, rtol, d));
                 bk_axpy_enabled<<<g2, 256, 0, ctx->stream>>>(dl, N, B.sys, gp.st, xQH);
@@ -1725,8 +2018,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
                   nc.max_refine = max_refine;
                   nc.max_iter = max_iter;
                   nc.incr = incr ? 1 : 0;
-                  bk_norm_then<<<dim3(S, gp.CH), 256, 0, ctx->stream>>>(r, N, h, B.off, gp, 1, nc);
-                  ++ctx->launches;
+                  launch_norm(ctx, B, h, gp, r, 1, nc);
                 }
                 GBI_CHECK(cudaGetLastError());
                 return gb.body(gb.node(hif, cudaGraphCondTypeIf), kBodyIf, [&]() -> gbi_status {
@@ -1858,8 +2150,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
     NormCtl nc{};
     nc.follow = follow;
     nc.rtol = rtol;
-    bk_norm_then<<<dim3(S, gp.CH), 256, 0, ctx->stream>>>(x, N, h, B.off, gp, mode, nc);
-    ++ctx->launches;
+    launch_norm(ctx, B, h, gp, x, mode, nc);
   };
   norm_refine(b, 2, kFollowRefine0);
   auto read_state = [&]() -> gbi_status {
