@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libgbi.so")
-SOURCES = ["gbi_api.cu", "common.cu", "solver.cu", "nearfield_api.cu", "trap_kernel.cu", "mlp_kernel.cu",
+SOURCES = ["gbi_api.cu", "common.cu", "solver.cu", "nearfield_api.cu", "trap_kernel.cu", "trap_steps.cu", "mlp_kernel.cu",
            "mlp_tc.cu", "flow.cu", "wall.cu", "periodic.cu"] + ["pairs_%s_%d.cu" % (p, t) for p in ("f32", "f64", "df") for t in (2, 3, 4)] + \
     ["pairs_f64_5.cu", "pairs_f64_40.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -186,6 +186,9 @@ bool balanced_args(gbi_ctx* ctx, int trunc, int rows, int precision, int N, Pair
 // scratch cannot be had
 bool split_reserve(gbi_ctx* ctx, int trunc, int rows, int precision, PairArgs& a);
 cudaError_t run_trap(gbi_ctx* ctx, const TrapArgs& t, int precision);
+// nsteps Euler steps of one suspension in a trap by the l <= 2 superposition in FP32 (trap_steps.cu)
+gbi_status superposition_steps(gbi_ctx* ctx, const gbi_params* prm, int N, double dt, double k_trap, double vs,
+                               double s0, double d0, int nsteps, double* R, double* p);
 int d_of(int trunc);
 const double* scale_tab(int trunc);
 const double* self_tab(int trunc);

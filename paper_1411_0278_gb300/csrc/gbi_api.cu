@@ -476,6 +476,15 @@ gbi_status trap_steps(gbi_ctx* ctx, const gbi_params* prm, int nsys, const int* 
     return GBI_OK;
   }
   if (!R || !p) return GBI_ERR_ARG;
+  if (superposition && offsets == nullptr && prm->trunc == 2 && (prm->precision == 1 || prm->precision == 3)) {
+    // one suspension, closed-form FP32 sums: kernels of their own (trap_steps.cu); FP64, l >= 3
+    // and batches take the general sequence below
+    GBI_TRY(superposition_steps(ctx, prm, N, dt, k_trap, vs, s0, d0, nsteps, R, p));
+    total.matvecs_f32 = nsteps;
+    total.pair_interactions = (long long)nsteps * N * (N - 1);
+    if (info) *info = total;
+    return GBI_OK;
+  }
   const int h = gbi_h(prm->trunc);
   GBI_TRY(ensure(ctx, ctx->tFe, sizeof(double) * 3 * N));
   GBI_TRY(ensure(ctx, ctx->tTe, sizeof(double) * 3 * N));

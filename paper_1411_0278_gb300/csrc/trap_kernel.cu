@@ -22,6 +22,7 @@
 #include <type_traits>
 
 #include "df.cuh"
+#include "f2.cuh"
 #include "gbi_generated.cuh"
 #include "gbi_internal.cuh"
 
@@ -135,24 +136,6 @@ __device__ __forceinline__ void trap_source(const T* __restrict__ s_rec, int j, 
     w2[t] = gbi_fmac(tx, Sy, gbi_fmac(-ty, Sx, gbi_fmac(ct, z, gbi_fmac(ri3, e2, w2[t]))));
   }
 }
-
-// Two FP32 values per instruction (the paired FFMA2 / FMUL2 / FADD2 of sm_100 and later).
-// Each element is rounded exactly as the scalar operation rounds it, so the paired pass
-// gives the scalar pass's results bit for bit; it halves the issued FP32 instructions,
-// not the FMA pipe's work (a paired FMA occupies the pipe for two lanes' worth).
-struct f2 {
-  float2 v;
-  __device__ __forceinline__ f2() {}
-  __device__ __forceinline__ explicit f2(float s) : v(make_float2(s, s)) {}
-  __device__ __forceinline__ f2(float a, float b) : v(make_float2(a, b)) {}
-  __device__ __forceinline__ explicit f2(float2 p) : v(p) {}
-};
-__device__ __forceinline__ f2 operator+(f2 a, f2 b) { return f2(__fadd2_rn(a.v, b.v)); }
-__device__ __forceinline__ f2 operator*(f2 a, f2 b) { return f2(__fmul2_rn(a.v, b.v)); }
-__device__ __forceinline__ f2 operator-(f2 a) { return f2(-a.v.x, -a.v.y); }
-__device__ __forceinline__ f2 operator-(f2 a, f2 b) { return a + (-b); }
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
-__device__ __forceinline__ f2 rsqrt2(f2 a) { return f2(rsqrtf(a.v.x), rsqrtf(a.v.y)); }
 
 // trap_source for FP32 targets taken two at a time: pair g holds targets n0 + 2g (x) and
 // n0 + 2g + 1 (y).  The source record sits in shared memory with every word duplicated
