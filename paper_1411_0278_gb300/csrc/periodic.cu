@@ -55,6 +55,7 @@
 #include <vector>
 
 #include "ctx.cuh"
+#include "f2.cuh"
 
 namespace gbi {
 namespace {
@@ -152,32 +153,48 @@ __device__ __forceinline__ double per_frac(const double* __restrict__ R, size_t 
   return sd;
 }
 
-// the cell key of every sphere (cells c_d = floor(M s_d)) and the identity permutation
+// the cell key of every sphere (cells c_d = floor(M s_d)), the identity permutation, and the
+// fractions s themselves: their FP64 divisions (some 20 instructions of 16 cycles each) are made
+// once here and not again by the records, the spreading and the gathering
 __global__ void k_per_keys(int N, double L, int M, const double* __restrict__ R, unsigned int* __restrict__ key,
-                           int* __restrict__ idx) {
+                           int* __restrict__ idx, double* __restrict__ frac) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   int c[3];
   for (int d = 0; d < 3; ++d) {
-    const int cd = (int)(per_frac(R, (size_t)n, d, L) * M);
+    const double s = per_frac(R, (size_t)n, d, L);
+    frac[3 * (size_t)n + d] = s;
+    const int cd = (int)(s * M);
     c[d] = cd < 0 ? 0 : (cd >= M ? M - 1 : cd);
   }
   key[n] = (unsigned int)(c[0] + M * (c[1] + M * c[2]));
   idx[n] = n;
 }
 
+// Where a record's force is spread on the mesh: first grid point k0 of each axis (u = K s, k0 =
+// floor(u), the points are k0 - j mod K) and the fraction u - k0
+template <typename G> struct alignas(4 * sizeof(G)) PmePoint {
+  G f[3];
+  int pad;
+  int k0[3];
+  int pad2;
+};
+
 // Record t (sphere n = order[t], or t without a sort): pos[16] = s_hi (3), 0, s_lo (3), 0,
-// s15 (3), 0, s_rem (3), 0 of the cell fraction s (FP64: s, 0, s, 0); frc[4] = F, 0.
+// s15 (3), 0, s_rem (3), 0 of the cell fraction s (FP64: s, 0, s, 0); frc[4] = F, 0; with a
+// mesh (K > 0) its point pt[t].
 template <typename T>
-__global__ void k_per_records(int N, double L, const double* __restrict__ R, const double* __restrict__ F,
-                              const int* __restrict__ order, T* __restrict__ pos, T* __restrict__ frc) {
+__global__ void k_per_records(int N, double L, const double* __restrict__ R, const double* __restrict__ frac,
+                              const double* __restrict__ F, const int* __restrict__ order, T* __restrict__ pos,
+                              T* __restrict__ frc, int K, PmePoint<T>* __restrict__ pt) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N) return;
   const size_t n = order ? (size_t)order[t] : (size_t)t;
   constexpr bool F32 = std::is_same<T, float>::value;
   T* o = pos + 16 * (size_t)t;
+  PmePoint<T> q;
   for (int d = 0; d < 3; ++d) {
-    const double sd = per_frac(R, n, d, L);
+    const double sd = frac ? frac[3 * n + d] : per_frac(R, n, d, L);
     if (F32) {
       const float hi = float(sd);
       const float s15 = float(floor(sd * 32768.0) / 32768.0);
@@ -192,9 +209,16 @@ __global__ void k_per_records(int N, double L, const double* __restrict__ R, con
       o[12 + d] = T(0);
     }
     frc[4 * (size_t)t + d] = T(F[3 * n + d]);
+    const double u = sd * K, fl = floor(u);
+    q.k0[d] = (int)fl;
+    q.f[d] = T(u - fl);
   }
   o[3] = o[7] = o[11] = o[15] = T(0);
   frc[4 * (size_t)t + 3] = T(0);
+  if (K > 0) {
+    q.pad = q.pad2 = 0;
+    pt[t] = q;
+  }
 }
 
 // first and one-past-last sorted position of every cell (cells start empty: 0, 0)
@@ -279,19 +303,56 @@ __device__ __forceinline__ void per_real_staged(const T* pn, const T* sp, const 
 // Real-space sums by cells (M >= 3, records in cell order).  blockIdx.x is the target
 // cell, blockIdx.y one of gridDim.y passes over its records, kPerCellSlots targets per pass.
 // The sources of the 27 cells around it (ranges of the cell order) are staged in shared
-// memory in chunks of up to kPerCellCap records; thread (slot, quarter) adds to target
-// `slot` the chunk's sources j = quarter (mod 4).  Sources are taken 32 at a time: first a
-// bit mask of those within the cut-off (r > 0 leaves the target itself out), then only
-// those are evaluated, so the lanes of a warp diverge only in how many.  The four quarters'
-// compensated sums are added at the end.
+// memory in chunks of up to kPerCellCap records, their high parts also shifted to the image
+// next to the target cell, so that the cut-off test wraps nothing (a rounding instruction per
+// coordinate, a quarter of the FMA rate); thread (slot, quarter) adds to target `slot` every
+// fourth batch of 32 of the chunk.
+// Batches are taken four at a time: first the bit masks of the sources within the cut-off (r > 0
+// leaves the target itself out; two sources per paired instruction in FP32, coordinates of four
+// per load), then only those are evaluated, so the lanes of a warp diverge only in how many of
+// 128 -- of 32 at a time the longest lane had twice the mean.  The four quarters' compensated sums
+// are added at the end.  Instruction issue bounds it: 15 % of the candidates are inside, a test
+// takes about 7 instructions and a term about 90.  N = 10^5: kRealUs.
 constexpr int kPerCellThreads = 256;
 constexpr int kPerCellSlots = 64;
 constexpr int kPerCellQuarters = kPerCellThreads / kPerCellSlots;
-template <typename T> struct PerCellCap { static constexpr int v = sizeof(T) == 4 ? 1024 : 512; };
+template <typename T> struct PerCellCap { static constexpr int v = sizeof(T) == 4 ? 896 : 448; };   // < 48 KB
 
 template <typename T> struct PerQuad;
 template <> struct PerQuad<float> { using t = float4; };
 template <> struct PerQuad<double> { using t = Dbl4; };
+
+// bit i of the result: source i of the 32 at x, y, z (aligned to 16 bytes) lies within the cut-off of
+// the target (box units), judged by the high parts alone (a pair it misjudges sits at r_c,
+// where its term is erfc(xi r_c) ~ 3e-9 of a near pair's); the target itself gives r2 = 0
+__device__ __forceinline__ unsigned int per_near(const float* x, const float* y, const float* z, const float* pn, float rc2) {
+  unsigned int mask = 0u;
+  const f2 px(pn[0]), py(pn[1]), pz(pn[2]);
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    const float4 qx = *reinterpret_cast<const float4*>(x + i), qy = *reinterpret_cast<const float4*>(y + i),
+                 qz = *reinterpret_cast<const float4*>(z + i);
+    const f2 ax = px - f2(qx.x, qx.y), ay = py - f2(qy.x, qy.y), az = pz - f2(qz.x, qz.y);
+    const f2 bx = px - f2(qx.z, qx.w), by = py - f2(qy.z, qy.w), bz = pz - f2(qz.z, qz.w);
+    const f2 ra = fma2(az, az, fma2(ay, ay, ax * ax)), rb = fma2(bz, bz, fma2(by, by, bx * bx));
+    if (ra.v.x < rc2 && ra.v.x > 0.f) mask |= 1u << i;
+    if (ra.v.y < rc2 && ra.v.y > 0.f) mask |= 2u << i;
+    if (rb.v.x < rc2 && rb.v.x > 0.f) mask |= 4u << i;
+    if (rb.v.y < rc2 && rb.v.y > 0.f) mask |= 8u << i;
+  }
+  return mask;
+}
+__device__ __forceinline__ unsigned int per_near(const double* x, const double* y, const double* z, const double* pn,
+                                                 double rc2) {
+  unsigned int mask = 0u;
+#pragma unroll 8
+  for (int i = 0; i < 32; ++i) {
+    const double a = pn[0] - x[i], b = pn[1] - y[i], c = pn[2] - z[i];
+    const double r2 = a * a + b * b + c * c;
+    if (r2 < rc2 && r2 > 0.0) mask |= 1u << i;
+  }
+  return mask;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kPerCellThreads)
@@ -299,21 +360,31 @@ __global__ void __launch_bounds__(kPerCellThreads)
                      const int* __restrict__ cstart, const int* __restrict__ cend, T* __restrict__ u_out) {
   using Q4 = typename PerQuad<T>::t;
   constexpr int kCap = PerCellCap<T>::v;
-  // source j: sa = (s_hi, F_x), sb = (s_lo, F_y), sc = F_z
+  // source j: shifted high parts sx, sy, sz; sa = (s_hi, F_x), sb = (s_lo, F_y), sc = F_z
+  __shared__ __align__(16) T sx[kCap], sy[kCap], sz[kCap];
   __shared__ Q4 sa[kCap], sb[kCap];
   __shared__ T sc[kCap];
-  __shared__ int r_start[27], r_pre[28];
+  __shared__ int r_start[27], r_pre[28], r_shift[27];
   __shared__ T red[kPerCellQuarters - 1][kPerCellSlots][3];
   const int cell = blockIdx.x;
   const int c[3] = {cell % M, (cell / M) % M, cell / (M * M)};
   const int t0 = cstart[cell], t1 = cend[cell];
+  if (t0 + blockIdx.y * kPerCellSlots >= t1) return;   // no targets in this pass
   if (threadIdx.x < 27) {
     const int o = threadIdx.x;
-    const int cx = (c[0] + o % 3 - 1 + M) % M, cy = (c[1] + (o / 3) % 3 - 1 + M) % M,
-              cz = (c[2] + o / 9 - 1 + M) % M;
-    const int nb = cx + M * (cy + M * cz);
+    int nb = 0, shift = 0;
+    const int d[3] = {o % 3 - 1, (o / 3) % 3 - 1, o / 9 - 1};
+#pragma unroll
+    for (int k = 2; k >= 0; --k) {
+      int x = c[k] + d[k], w = 0;
+      if (x < 0) { x += M; w = -1; }
+      if (x >= M) { x -= M; w = 1; }
+      nb = nb * M + x;
+      shift = shift * 3 + (w + 1);
+    }
     r_start[o] = cstart[nb];
     r_pre[o + 1] = cend[nb] - cstart[nb];
+    r_shift[o] = shift;   // base 3: x least significant
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -324,6 +395,7 @@ __global__ void __launch_bounds__(kPerCellThreads)
   const int total = r_pre[27];
   const int slot = threadIdx.x % kPerCellSlots, quarter = threadIdx.x / kPerCellSlots;
   const T Lt = T(L), rc2 = T(rc * rc), xit = T(xi);
+  const T rc2u = T((rc / L) * (rc / L));
   for (int tp = t0 + blockIdx.y * kPerCellSlots; tp < t1; tp += gridDim.y * kPerCellSlots) {
     const int t = tp + slot;
     const bool live = t < t1;
@@ -335,15 +407,11 @@ __global__ void __launch_bounds__(kPerCellThreads)
     }
     T u[3] = {T(0), T(0), T(0)}, uc[3] = {T(0), T(0), T(0)};
     for (int base = 0; base < total; base += kCap) {
-      const int n = min(kCap, total - base);
+      const int n = min(kCap, total - base), npad = (n + 31) & ~31;
       __syncthreads();   // the previous chunk is done
-      // stage records base .. base + n - 1 of the 27 ranges (loads issued together)
-      constexpr int kPer = kCap / kPerCellThreads;
-      Q4 la[kPer], lb[kPer];
-      T lc[kPer];
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const int e = threadIdx.x + k * kPerCellThreads;
+      // stage records base .. base + n - 1 of the 27 ranges; the last batch is filled up with
+      // far points
+      for (int e = threadIdx.x; e < npad; e += kPerCellThreads) {
         if (e < n) {
           const int g = base + e;
           int o = 0;
@@ -351,45 +419,39 @@ __global__ void __launch_bounds__(kPerCellThreads)
           const size_t m = (size_t)(r_start[o] + (g - r_pre[o]));
           const T* pm = pos + 16 * m;
           const T* fm = frc + 4 * m;
-          la[k] = Q4{pm[0], pm[1], pm[2], fm[0]};
-          lb[k] = Q4{pm[4], pm[5], pm[6], fm[1]};
-          lc[k] = fm[2];
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const int e = threadIdx.x + k * kPerCellThreads;
-        if (e < n) {
-          sa[e] = la[k];
-          sb[e] = lb[k];
-          sc[e] = lc[k];
+          const int sh = r_shift[o];
+          sa[e] = Q4{pm[0], pm[1], pm[2], fm[0]};
+          sb[e] = Q4{pm[4], pm[5], pm[6], fm[1]};
+          sc[e] = fm[2];
+          sx[e] = pm[0] + T(sh % 3 - 1);
+          sy[e] = pm[1] + T((sh / 3) % 3 - 1);
+          sz[e] = pm[2] + T(sh / 9 - 1);
+        } else {
+          sx[e] = sy[e] = sz[e] = T(1e6);
         }
       }
       __syncthreads();
       if (!live) continue;
-      const int ni = (n - quarter + kPerCellQuarters - 1) / kPerCellQuarters;   // j = quarter + 4 i
-      for (int ib = 0; ib < ni; ib += 32) {
-        unsigned int mask = 0u;
-        // the cut-off test on the high parts alone (a pair it misjudges sits at r_c, where
-        // its term is erfc(xi r_c) ~ 3e-9 of a near pair's); the target itself gives r2 = 0
+      const int nb = npad >> 5;
+      for (int b0 = quarter; b0 < nb; b0 += 4 * kPerCellQuarters) {
+        unsigned int mk[4];
 #pragma unroll
-        for (int bit = 0; bit < 32; ++bit) {
-          const int i = ib + bit;
-          if (i < ni) {
-            const int j = quarter + kPerCellQuarters * i;
-            const Q4 qa = sa[j];
-            T v0 = pn[0] - qa.x, v1 = pn[1] - qa.y, v2 = pn[2] - qa.z;
-            v0 = (v0 - per_rint(v0)) * Lt;
-            v1 = (v1 - per_rint(v1)) * Lt;
-            v2 = (v2 - per_rint(v2)) * Lt;
-            const T r2 = v0 * v0 + v1 * v1 + v2 * v2;
-            mask |= (r2 < rc2 && r2 > T(0) ? 1u : 0u) << bit;
-          }
+        for (int q = 0; q < 4; ++q) {
+          const int b = b0 + q * kPerCellQuarters;
+          mk[q] = b < nb ? per_near(sx + 32 * b, sy + 32 * b, sz + 32 * b, pn, rc2u) : 0u;
         }
-        while (mask) {
-          const int bit = __ffs(mask) - 1;
-          mask &= mask - 1u;
-          const int j = quarter + kPerCellQuarters * (ib + bit);
+        int q = 0;
+        unsigned int cur = mk[0];
+        while (true) {
+          if (cur == 0u) {
+            do {
+              ++q;
+              cur = q == 1 ? mk[1] : (q == 2 ? mk[2] : (q == 3 ? mk[3] : 0u));
+            } while (cur == 0u && q < 4);
+            if (q >= 4) break;
+          }
+          const int j = 32 * (b0 + q * kPerCellQuarters) + __ffs(cur) - 1;
+          cur &= cur - 1u;
           const Q4 qa = sa[j], qb = sb[j];
           T v0 = (pn[0] - qa.x) + (pn[4] - qb.x), v1 = (pn[1] - qa.y) + (pn[5] - qb.y),
             v2 = (pn[2] - qa.z) + (pn[6] - qb.z);
@@ -575,23 +637,6 @@ template <typename G> __device__ __forceinline__ void pme_weights(G f, G* w) {
   }
 }
 
-// grid coordinate u = K s of a position (s the cell fraction in [0, 1)): first point k0
-// (the points are k0 - j mod K) and the spline weights of each axis
-template <typename G>
-__device__ __forceinline__ void pme_point(const double* __restrict__ R, size_t n, double L, int K, int* k0,
-                                          G (*w)[kPmeOrder]) {
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    double s = R[3 * n + d] / L;
-    s -= floor(s);
-    if (!(s < 1.0)) s = 0.0;
-    const double u = s * K;
-    const double fl = floor(u);
-    k0[d] = (int)fl;
-    pme_weights<G>(G(u - fl), w[d]);
-  }
-}
-
 __device__ __forceinline__ int pme_wrap(int g, int K) { return g < 0 ? g + K : g; }   // g > -K
 
 // Spreading, in the order of the cell sort (neighbouring threads touch neighbouring
@@ -610,30 +655,42 @@ __device__ __forceinline__ void pme_add(Dbl4* q, double wx, double wy, double wz
 // runs of eight neighbouring points)
 constexpr int kPmeLanes = kPmeOrder;
 
+// a lane's spline weights (its own along x, all along y and z) and the wrapped grid offsets
+template <typename G> struct PmeLane {
+  G wx, wy[kPmeOrder], wz[kPmeOrder];
+  unsigned int gx, gy[kPmeOrder], gz[kPmeOrder];   // gy = K y, gz = K^2 z
+  __device__ __forceinline__ PmeLane(const PmePoint<G>& p, int jx, int K) {
+    G w[kPmeOrder];
+    pme_weights<G>(p.f[0], w);
+    wx = w[0];
+#pragma unroll
+    for (int j = 1; j < kPmeOrder; ++j)
+      if (j == jx) wx = w[j];
+    pme_weights<G>(p.f[1], wy);
+    pme_weights<G>(p.f[2], wz);
+    gx = pme_wrap(p.k0[0] - jx, K);
+#pragma unroll
+    for (int j = 0; j < kPmeOrder; ++j) {
+      gy[j] = (unsigned)K * (unsigned)pme_wrap(p.k0[1] - j, K);
+      gz[j] = (unsigned)K * (unsigned)K * (unsigned)pme_wrap(p.k0[2] - j, K);
+    }
+  }
+};
+
 template <typename G>
-__global__ void k_pme_spread(int N, int K, const double* __restrict__ R, double L, const double* __restrict__ F,
-                             const int* __restrict__ order, typename Cplx<G>::q* __restrict__ Q) {
+__global__ void k_pme_spread(int N, int K, const PmePoint<G>* __restrict__ pt, const G* __restrict__ frc,
+                             typename Cplx<G>::q* __restrict__ Q) {
   const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int t = (int)(gt / kPmeLanes), jx = (int)(gt % kPmeLanes);
   if (t >= N) return;
-  const int n = order[t];
-  int k0[3];
-  G w[3][kPmeOrder];
-  pme_point<G>(R, (size_t)n, L, K, k0, w);
-  G wx = w[0][0];
-#pragma unroll
-  for (int j = 1; j < kPmeOrder; ++j)
-    if (j == jx) wx = w[0][j];
-  const G Fx = G(F[3 * (size_t)n]) * wx, Fy = G(F[3 * (size_t)n + 1]) * wx, Fz = G(F[3 * (size_t)n + 2]) * wx;
-  const size_t gx = (size_t)pme_wrap(k0[0] - jx, K);
+  const PmeLane<G> l(pt[t], jx, K);
+  const G Fx = frc[4 * (size_t)t] * l.wx, Fy = frc[4 * (size_t)t + 1] * l.wx, Fz = frc[4 * (size_t)t + 2] * l.wx;
 #pragma unroll
   for (int jz = 0; jz < kPmeOrder; ++jz) {
-    const size_t gz = (size_t)pme_wrap(k0[2] - jz, K);
 #pragma unroll
     for (int jy = 0; jy < kPmeOrder; ++jy) {
-      const size_t row = (size_t)K * ((size_t)pme_wrap(k0[1] - jy, K) + (size_t)K * gz);
-      const G wyz = w[1][jy] * w[2][jz];
-      pme_add(&Q[row + gx], wyz * Fx, wyz * Fy, wyz * Fz);
+      const G wyz = l.wy[jy] * l.wz[jz];
+      pme_add(&Q[l.gz[jz] + l.gy[jy] + l.gx], wyz * Fx, wyz * Fy, wyz * Fz);
     }
   }
 }
@@ -693,7 +750,17 @@ __device__ __forceinline__ void pme_reg_fft(C* v) {
         const int t = k * (16 / Ns);   // e^{-+2 pi i k / (2 Ns)} = e^{-+2 pi i t / 32}
         const G wc = G(pme_c32(t)), ws = INV ? G(pme_s32(t)) : G(-pme_s32(t));
         const C x0 = a[j], y = a[j + N / 2];
-        const G x1r = wc * y.x - ws * y.y, x1i = wc * y.y + ws * y.x;
+        G x1r, x1i;   // w y; the factors 1 and -+i without their products with 0 and 1
+        if (t == 0) {
+          x1r = y.x;
+          x1i = y.y;
+        } else if (t == 8) {
+          x1r = INV ? -y.y : y.y;
+          x1i = INV ? y.x : -y.x;
+        } else {
+          x1r = wc * y.x - ws * y.y;
+          x1i = wc * y.y + ws * y.x;
+        }
         const int o = (j - k) * 2 + k;
         b[o] = C{x0.x + x1r, x0.y + x1i};
         b[o + Ns] = C{x0.x - x1r, x0.y - x1i};
@@ -709,41 +776,57 @@ __device__ __forceinline__ void pme_reg_fft(C* v) {
 __host__ __device__ constexpr int pme_pad(int i) { return i + (i >> 4); }
 __host__ __device__ constexpr int pme_row(int K) { return K + K / 16 + 1; }
 
+// lines per FFT block (a function of K and the type, so that every index below is a shift and
+// every offset of an unrolled access a constant): at most 36 KB of padded rows (plus K twiddles),
+// at most 32 lines, dividing K, LB K within the elements a block holds
+template <typename G> __host__ __device__ constexpr int pme_lines(int K) {
+  int lb = 1;
+  while (lb < 32 && lb * 2 <= K && (size_t)(lb * 2) * pme_row(K) * 2 * sizeof(G) <= 36864 &&
+         lb * 2 * K <= pme_max_line_elems<G>())
+    lb *= 2;
+  return lb;
+}
+
 // The four-step transform of LB padded rows of K = 16 N2 values in shared memory (twf the
-// K twiddles e^{-+2 pi i t / K}, conjugated for the inverse); barriers inside.
-template <typename G, int N2, bool INV>
-__device__ __forceinline__ void pme_fft4_rows(typename Cplx<G>::t* sx, const typename Cplx<G>::t* twf, int LB) {
+// K twiddles e^{-+2 pi i t / K}, conjugated for the inverse); barriers inside.  pme_pad(x + c) =
+// pme_pad(x) + pme_pad(c) wherever x mod 16 + c mod 16 < 16, which holds for the power-of-two
+// strides here: an access is one base and a constant.
+template <typename G, int N2, int LB, bool INV>
+__device__ __forceinline__ void pme_fft4_rows(typename Cplx<G>::t* sx, const typename Cplx<G>::t* twf) {
   using C = typename Cplx<G>::t;
   constexpr int K = 16 * N2, RS = pme_row(K);
   // stage 1: task (row, n2)
-  for (int task = threadIdx.x; task < LB * N2; task += blockDim.x) {
-    const int lane = task / N2, n2 = task - lane * N2;
-    C* row = sx + lane * RS;
-    C v[16];
 #pragma unroll
-    for (int n1 = 0; n1 < 16; ++n1) v[n1] = row[pme_pad(N2 * n1 + n2)];
-    pme_reg_fft<C, 16, INV>(v);
+  for (int task0 = 0; task0 < LB * N2; task0 += kPmeFftThreads) {
+    const int task = task0 + threadIdx.x;
+    if (LB * N2 % kPmeFftThreads == 0 || task < LB * N2) {
+      const int n2 = task & (N2 - 1);
+      C* row = sx + (task / N2) * RS + pme_pad(n2);
+      C v[16];
 #pragma unroll
-    for (int k1 = 1; k1 < 16; ++k1) {
-      const C w = twf[n2 * k1];
-      const C a = v[k1];
-      v[k1] = C{w.x * a.x - w.y * a.y, w.x * a.y + w.y * a.x};
+      for (int n1 = 0; n1 < 16; ++n1) v[n1] = row[pme_pad(N2 * n1)];
+      pme_reg_fft<C, 16, INV>(v);
+#pragma unroll
+      for (int k1 = 1; k1 < 16; ++k1) {
+        const C w = twf[n2 * k1];
+        const C a = v[k1];
+        v[k1] = C{w.x * a.x - w.y * a.y, w.x * a.y + w.y * a.x};
+      }
+#pragma unroll
+      for (int k1 = 0; k1 < 16; ++k1) row[pme_pad(N2 * k1)] = v[k1];
     }
-#pragma unroll
-    for (int k1 = 0; k1 < 16; ++k1) row[pme_pad(N2 * k1 + n2)] = v[k1];
   }
   __syncthreads();
   // stage 2: task (row, k1), read everything before anything is written
-  constexpr int kT = (16 * 4096 / K + kPmeFftThreads - 1) / kPmeFftThreads;   // tasks per thread at most
+  constexpr int kT = (16 * LB + kPmeFftThreads - 1) / kPmeFftThreads;   // tasks per thread
   C u[kT][N2];
 #pragma unroll
   for (int t = 0; t < kT; ++t) {
     const int task = threadIdx.x + t * kPmeFftThreads;
-    if (task < LB * 16) {
-      const int lane = task >> 4, k1 = task & 15;
-      const C* row = sx + lane * RS;
+    if (16 * LB % kPmeFftThreads == 0 || task < LB * 16) {
+      const C* row = sx + (task >> 4) * RS + pme_pad(N2 * (task & 15));
 #pragma unroll
-      for (int n2 = 0; n2 < N2; ++n2) u[t][n2] = row[pme_pad(N2 * k1 + n2)];
+      for (int n2 = 0; n2 < N2; ++n2) u[t][n2] = row[pme_pad(n2)];
       pme_reg_fft<C, N2, INV>(u[t]);
     }
   }
@@ -751,98 +834,70 @@ __device__ __forceinline__ void pme_fft4_rows(typename Cplx<G>::t* sx, const typ
 #pragma unroll
   for (int t = 0; t < kT; ++t) {
     const int task = threadIdx.x + t * kPmeFftThreads;
-    if (task < LB * 16) {
-      const int lane = task >> 4, k1 = task & 15;
-      C* row = sx + lane * RS;
+    if (16 * LB % kPmeFftThreads == 0 || task < LB * 16) {
+      C* row = sx + (task >> 4) * RS + (task & 15);
 #pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) row[pme_pad(k1 + 16 * k2)] = u[t][k2];
+      for (int k2 = 0; k2 < N2; ++k2) row[pme_pad(16 * k2)] = u[t][k2];
     }
   }
   __syncthreads();
 }
 
-// In-place FFT of the K-point lines of one axis (K = 16 N2 <= 512), unnormalised,
-// e^{-2 pi i m g / K} (forward) or e^{+2 pi i m g / K} (inverse), natural order in and out.
-// The K^2 lines of a grid are numbered l = a + K b over the two other axes; line l holds
-//   axis 0: K l + i,   axis 1: a + K^2 b + K i,   axis 2: l + K^2 i   (i = 0..K-1).
-// A block transforms LB = 2^logLB consecutive lines (LB | K, LB K <= 4096 in FP32, 2048 in
-// FP64) in shared memory; consecutive lines are adjacent in memory along axes 1 and 2, so
-// those loads coalesce in runs of LB elements.  grids = A (blockIdx.y = 0) and B (1); with
-// src the lines are read from the staging points instead (A = x + i y, B = z).
-// tw[t] = e^{-2 pi i t / K}, t < K.  Indices are 32-bit (K^3 <= 2^27).
-template <typename G, int N2>
+// In-place FFT of the K-point lines of the y axis (AXIS 1) or z axis (2), K = 16 N2 <= 512,
+// unnormalised, e^{-2 pi i m g / K} (forward) or e^{+2 pi i m g / K} (INV), natural order in
+// and out.  The K^2 lines of a grid are numbered l = a + K b over the two other axes; line l holds
+//   axis 1: a + K^2 b + K i,   axis 2: l + K^2 i   (i = 0..K-1).
+// A block transforms LB consecutive lines in shared memory; they are adjacent in memory, so the
+// loads coalesce in runs of LB elements.  grids = A (blockIdx.y = 0) and B (1); with SRC the
+// lines are read from the staging points instead (A = x + i y, B = z).  tw[t] = e^{-2 pi i t / K},
+// t < K.  Indices are 32-bit (K^3 <= 2^27).  Axis, direction and lines are template parameters:
+// with them as arguments two thirds of the ~106 instructions per element were index arithmetic
+// (ncu: issue 63 % active, FMA pipe 21 %).  K = 256: kFftUs a pass.
+template <typename G, int N2, int AXIS, bool INV, bool SRC>
 __global__ void __launch_bounds__(kPmeFftThreads, (sizeof(G) == 4 && N2 >= 16) ? 3 : 1)
-    k_pme_fft4(typename Cplx<G>::t* __restrict__ grids, const typename Cplx<G>::q* __restrict__ src, int logLB,
-               int axis, int inverse, const typename Cplx<G>::t* __restrict__ tw) {
+    k_pme_fft4(typename Cplx<G>::t* __restrict__ grids, const typename Cplx<G>::q* __restrict__ src,
+               const typename Cplx<G>::t* __restrict__ tw) {
   using C = typename Cplx<G>::t;
-  constexpr int K = 16 * N2, RS = pme_row(K), logK = pme_log2(K);
+  constexpr int K = 16 * N2, RS = pme_row(K), logK = pme_log2(K), LB = pme_lines<G>(K), logLB = pme_log2(LB);
+  constexpr unsigned int K2 = (unsigned)K * K, S = AXIS == 1 ? (unsigned)K : K2;
   extern __shared__ __align__(16) unsigned char pme_smem[];
   C* sx = reinterpret_cast<C*>(pme_smem);
-  const int LB = 1 << logLB;
   C* stw = sx + (size_t)LB * RS;
-  const unsigned int K2 = (unsigned)K * K;
   C* g = grids + (size_t)blockIdx.y * K2 * K;
-  const unsigned int l0 = blockIdx.x << logLB;
-  const unsigned int tot = (unsigned)LB * K;
   for (unsigned int j = threadIdx.x; j < (unsigned)K; j += blockDim.x) {
     C w = tw[j];
-    if (inverse) w.y = -w.y;
+    if (INV) w.y = -w.y;
     stw[j] = w;
   }
-  auto at = [&](unsigned int e, unsigned int& si) -> unsigned int {
-    unsigned int lane, i;
-    if (axis == 0) {
-      lane = e >> logK;
-      i = e & (K - 1u);
-      si = lane * RS + pme_pad((int)i);
-      return ((l0 + lane) << logK) + i;
-    }
-    lane = e & ((unsigned)LB - 1u);
-    i = e >> logLB;
-    si = lane * RS + pme_pad((int)i);
-    const unsigned int l = l0 + lane;
-    if (axis == 1) return (l & (K - 1u)) + ((l >> logK) << (2 * logK)) + (i << logK);
-    return l + (i << (2 * logK));
-  };
-  constexpr int kMaxE = pme_max_line_elems<G>() / kPmeFftThreads;
-  C v[kMaxE];
+  // thread: line l0 + lane, elements i0 + k step
+  constexpr unsigned int step = kPmeFftThreads / LB, tot = (unsigned)LB * K;
+  constexpr int kE = (int)((tot + kPmeFftThreads - 1) / kPmeFftThreads);
+  const unsigned int lane = threadIdx.x & (LB - 1u), i0 = threadIdx.x >> logLB;
+  const unsigned int l = blockIdx.x * LB + lane;
+  const unsigned int ad = (AXIS == 1 ? (l & (K - 1u)) + ((l >> logK) << (2 * logK)) : l) + i0 * S;
+  C* sl = sx + lane * RS + pme_pad((int)i0);
+  C v[kE];
+  if (SRC) {
+    const typename Cplx<G>::q* q = src + ad;
+    const bool first = blockIdx.y == 0;
 #pragma unroll
-  for (int k = 0; k < kMaxE; ++k) {
-    const unsigned int e = threadIdx.x + k * kPmeFftThreads;
-    if (e < tot) {
-      unsigned int si;
-      const unsigned int ad = at(e, si);
-      if (src) {
-        const typename Cplx<G>::q q = src[ad];
-        v[k] = blockIdx.y == 0 ? C{q.x, q.y} : C{q.z, G(0)};
-      } else {
-        v[k] = g[ad];
-      }
+    for (int k = 0; k < kE; ++k) {
+      const G* w = reinterpret_cast<const G*>(q + (size_t)k * step * S);
+      if (first) v[k] = *reinterpret_cast<const C*>(w);
+      else v[k] = C{w[2], G(0)};
     }
+  } else {
+    const C* q = g + ad;
+#pragma unroll
+    for (int k = 0; k < kE; ++k) v[k] = q[(size_t)k * step * S];
   }
 #pragma unroll
-  for (int k = 0; k < kMaxE; ++k) {
-    const unsigned int e = threadIdx.x + k * kPmeFftThreads;
-    if (e < tot) {
-      unsigned int si;
-      at(e, si);
-      sx[si] = v[k];
-    }
-  }
+  for (int k = 0; k < kE; ++k) sl[pme_pad((int)(k * step))] = v[k];
   __syncthreads();
-  if (inverse)
-    pme_fft4_rows<G, N2, true>(sx, stw, LB);
-  else
-    pme_fft4_rows<G, N2, false>(sx, stw, LB);
+  pme_fft4_rows<G, N2, LB, INV>(sx, stw);
+  C* q = g + ad;
 #pragma unroll
-  for (int k = 0; k < kMaxE; ++k) {
-    const unsigned int e = threadIdx.x + k * kPmeFftThreads;
-    if (e < tot) {
-      unsigned int si;
-      const unsigned int ad = at(e, si);
-      g[ad] = sx[si];
-    }
-  }
+  for (int k = 0; k < kE; ++k) q[(size_t)k * step * S] = sl[pme_pad((int)(k * step))];
 }
 
 // Wave space on the mesh, fused with the transforms along x.  On entry A = FT_yz(Q_x + i Q_y)
@@ -859,15 +914,15 @@ __global__ void __launch_bounds__(kPmeFftThreads, (sizeof(G) == 4 && N2 >= 16) ?
 // A(m) = U_x + i U_y, B(m) = U_z (the mirror -m lies in the mirror row at (K - i) mod K), then
 // transforms back along x and stores the rows it owns.  bmod[i] = |b_i|^2 of one axis.
 template <typename G, int N2>
-__global__ void __launch_bounds__(kPmeFftThreads)
-    k_pme_xconv(typename Cplx<G>::t* __restrict__ A, typename Cplx<G>::t* __restrict__ B, int logP, double L,
-                double xi, const G* __restrict__ bmod, const typename Cplx<G>::t* __restrict__ tw) {
+__global__ void __launch_bounds__(kPmeFftThreads, (sizeof(G) == 4 && N2 >= 16) ? 3 : 1)
+    k_pme_xconv(typename Cplx<G>::t* __restrict__ A, typename Cplx<G>::t* __restrict__ B, G s, G c0, G cq,
+                const G* __restrict__ bmod, const typename Cplx<G>::t* __restrict__ tw) {
   using C = typename Cplx<G>::t;
   extern __shared__ __align__(16) unsigned char pme_smem[];
   constexpr int RS = pme_row(16 * N2), logK = pme_log2(16 * N2);
-  const unsigned int K = 16u * N2, mask = K - 1u, P = 1u << logP;
-  const int logLB = logP + 2;   // rows: A own, A mirror, B own, B mirror
-  const int LB = 1 << logLB;
+  // rows: A own, A mirror, B own, B mirror, P of each
+  constexpr int LB = pme_lines<G>(16 * N2), logLB = pme_log2(LB), logP = logLB - 2;
+  constexpr unsigned int K = 16u * N2, mask = K - 1u, P = 1u << logP;
   C* sx = reinterpret_cast<C*>(pme_smem);
   C* stw = sx + (size_t)LB * RS;
   const unsigned int r0 = blockIdx.x << logP;
@@ -888,8 +943,8 @@ __global__ void __launch_bounds__(kPmeFftThreads)
     return g + ((size_t)(mir ? mir_row(sl) : own_row(sl)) << logK);
   };
   for (unsigned int j = threadIdx.x; j < K; j += blockDim.x) stw[j] = tw[j];
-  const unsigned int tot = 1u << (logLB + logK);
-  constexpr int kMaxE = pme_max_line_elems<G>() / kPmeFftThreads;
+  constexpr unsigned int tot = 1u << (logLB + logK);
+  constexpr int kMaxE = (int)((tot + kPmeFftThreads - 1) / kPmeFftThreads);
   C v[kMaxE];
 #pragma unroll
   for (int k = 0; k < kMaxE; ++k) {
@@ -902,14 +957,13 @@ __global__ void __launch_bounds__(kPmeFftThreads)
     if (e < tot) sx[(e >> logK) * RS + pme_pad((int)(e & mask))] = v[k];
   }
   __syncthreads();
-  pme_fft4_rows<G, N2, false>(sx, stw, LB);
+  pme_fft4_rows<G, N2, LB, false>(sx, stw);
   // the products: element e of the A rows (own and mirror) and the same element of B
-  const G s = G(2.0 * kPi / L);
-  const G c0 = G(8.0 * kPi / (L * L * L)), cq = G(0.25 / (xi * xi));
-  const unsigned int ntot = 1u << (logP + 1 + logK);   // A own and mirror rows
-  C ua[kMaxE / 2], ub[kMaxE / 2];
+  constexpr unsigned int ntot = 1u << (logP + 1 + logK);   // A own and mirror rows
+  constexpr int kHalf = (kMaxE + 1) / 2;
+  C ua[kHalf], ub[kHalf];
 #pragma unroll
-  for (int k = 0; k < kMaxE / 2; ++k) {
+  for (int k = 0; k < kHalf; ++k) {
     const unsigned int e = threadIdx.x + k * kPmeFftThreads;
     if (e < ntot) {
       const unsigned int q = e >> logK, ix = e & mask;
@@ -947,7 +1001,7 @@ __global__ void __launch_bounds__(kPmeFftThreads)
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < kMaxE / 2; ++k) {
+  for (int k = 0; k < kHalf; ++k) {
     const unsigned int e = threadIdx.x + k * kPmeFftThreads;
     if (e < ntot) {
       const unsigned int q = e >> logK, ix = e & mask;
@@ -958,7 +1012,7 @@ __global__ void __launch_bounds__(kPmeFftThreads)
   __syncthreads();
   for (unsigned int j = threadIdx.x; j < K; j += blockDim.x) stw[j].y = -stw[j].y;   // the inverse's twiddles
   __syncthreads();
-  pme_fft4_rows<G, N2, true>(sx, stw, LB);
+  pme_fft4_rows<G, N2, LB, true>(sx, stw);
   // store the rows this block owns: own rows of active slots, mirror rows of active slots
   // that are not their own mirror
 #pragma unroll
@@ -978,31 +1032,22 @@ __global__ void __launch_bounds__(kPmeFftThreads)
 // real and imaginary parts of A, u_z the real part of B), and the final velocities
 // V = Va + F / (6 pi eta a) + (u_real + u_wave - 8 xi / sqrt(pi) F) / (8 pi eta)
 template <typename G, typename T>
-__global__ void k_pme_gather(int N, int K, const double* __restrict__ R, double L, const double* __restrict__ F,
+__global__ void k_pme_gather(int N, int K, const PmePoint<G>* __restrict__ pt, const double* __restrict__ F,
                              const int* __restrict__ order, const typename Cplx<G>::t* __restrict__ A,
-                             const typename Cplx<G>::t* __restrict__ B, double xi, double a, double eta,
+                             const typename Cplx<G>::t* __restrict__ B, double self, double mob, double gg,
                              const T* __restrict__ u_real, const double* __restrict__ Va, double* __restrict__ V) {
   const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int t = (int)(gt / kPmeLanes), jx = (int)(gt % kPmeLanes);
   const bool live = t < N;   // the eight lanes of a sphere are live or not together
-  const int n = live ? order[t] : 0;
   G u[3] = {G(0), G(0), G(0)}, uc[3] = {G(0), G(0), G(0)};
   if (live) {
-    int k0[3];
-    G w[3][kPmeOrder];
-    pme_point<G>(R, (size_t)n, L, K, k0, w);
-    G wx = w[0][0];
-#pragma unroll
-    for (int j = 1; j < kPmeOrder; ++j)
-      if (j == jx) wx = w[0][j];
-    const size_t gx = (size_t)pme_wrap(k0[0] - jx, K);
+    const PmeLane<G> l(pt[t], jx, K);
 #pragma unroll
     for (int jz = 0; jz < kPmeOrder; ++jz) {
-      const size_t gz = (size_t)pme_wrap(k0[2] - jz, K);
 #pragma unroll
       for (int jy = 0; jy < kPmeOrder; ++jy) {
-        const size_t g = (size_t)K * ((size_t)pme_wrap(k0[1] - jy, K) + (size_t)K * gz) + gx;
-        const G ww = wx * w[1][jy] * w[2][jz];
+        const unsigned int g = l.gz[jz] + l.gy[jy] + l.gx;
+        const G ww = l.wx * l.wy[jy] * l.wz[jz];
         const typename Cplx<G>::t av = A[g];
         per_add(u[0], uc[0], ww * av.x);
         per_add(u[1], uc[1], ww * av.y);
@@ -1017,14 +1062,13 @@ __global__ void k_pme_gather(int N, int K, const double* __restrict__ R, double 
 #pragma unroll
     for (int off = kPmeLanes / 2; off > 0; off >>= 1) u[d] += __shfl_xor_sync(0xffffffffu, u[d], off);
   }
-  if (!live || jx != 0) return;
-  const double self = 8.0 * xi / kSqrtPi;
-  const double mob = 1.0 / (6.0 * kPi * eta * a), gg = 1.0 / (8.0 * kPi * eta);
-  for (int d = 0; d < 3; ++d) {
-    const double f = F[3 * (size_t)n + d];
-    const double un = double(u_real[3 * (size_t)t + d]) + double(u[d]) - self * f;   // record t
-    V[3 * (size_t)n + d] = Va[3 * (size_t)n + d] + mob * f + gg * un;
-  }
+  if (!live || jx >= 3) return;
+  // lane d finishes component d (an FP64 instruction costs a warp the same for one lane or all);
+  // self = 8 xi / sqrt(pi), mob = 1 / (6 pi eta a), gg = 1 / (8 pi eta)
+  const size_t n = (size_t)order[t];
+  const double f = F[3 * n + jx];
+  const double un = double(u_real[3 * (size_t)t + jx]) + double(jx == 0 ? u[0] : (jx == 1 ? u[1] : u[2])) - self * f;
+  V[3 * n + jx] = Va[3 * n + jx] + mob * f + gg * un;
 }
 
 // |b(m)|^2 = 1 / |sum_{j=0}^{p-2} M_p(j + 1) e^{2 pi i m j / K}|^2 for m = 0..K-1 (the
@@ -1053,23 +1097,14 @@ std::vector<double> pme_bmod(int K) {
   return out;
 }
 
-// lines per FFT block: at most 36 KB of padded rows (plus K twiddles), at most 32, at least
-// 4 (the fused x kernel's row quartets), dividing K, LB K within the elements a block holds
-int pme_lines_per_block(int K, size_t elem) {
-  const int cap = elem == sizeof(float2) ? 4096 : 2048;
-  int lb = 1;
-  while (lb < 32 && lb * 2 <= K && (size_t)(lb * 2) * pme_row(K) * elem <= 36864 && lb * 2 * K <= cap) lb *= 2;
-  return lb;
-}
-
 size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 struct PerBufs {
-  size_t o_pos, o_frc, o_ur, o_kv, o_S, o_key, o_skey, o_idx, o_sidx, o_cs, o_ce, o_tmp, o_grid, total;
+  size_t o_pos, o_frc, o_ur, o_kv, o_S, o_key, o_skey, o_idx, o_sidx, o_cs, o_ce, o_frac, o_pt, o_tmp, o_grid, total;
 };
 
 template <typename T>
-PerBufs per_layout(int N, long long nk, size_t ncell, size_t sort_bytes, size_t grid_bytes) {
+PerBufs per_layout(int N, long long nk, size_t ncell, size_t sort_bytes, size_t grid_bytes, bool sorted) {
   PerBufs o;
   o.o_pos = 0;
   o.o_frc = o.o_pos + al256(sizeof(T) * 16 * (size_t)N);
@@ -1082,7 +1117,9 @@ PerBufs per_layout(int N, long long nk, size_t ncell, size_t sort_bytes, size_t 
   o.o_sidx = o.o_idx + al256(sizeof(int) * (size_t)N);
   o.o_cs = o.o_sidx + al256(sizeof(int) * (size_t)N);
   o.o_ce = o.o_cs + al256(sizeof(int) * ncell);
-  o.o_tmp = o.o_ce + al256(sizeof(int) * ncell);
+  o.o_frac = o.o_ce + al256(sizeof(int) * ncell);
+  o.o_pt = o.o_frac + al256(sorted ? sizeof(double) * 3 * (size_t)N : 1);
+  o.o_tmp = o.o_pt + al256(grid_bytes > 0 ? sizeof(PmePoint<T>) * (size_t)N : 1);
   o.o_grid = o.o_tmp + al256(sort_bytes + 1);
   o.total = o.o_grid + al256(grid_bytes + 1);
   return o;
@@ -1100,9 +1137,11 @@ gbi_status run_periodic(gbi_ctx* ctx, int N, double L, double a, double eta, con
   const int M = p.M;
   const size_t ncell = M > 0 ? (size_t)M * M * M : 1;
   size_t sort_bytes = 0;
+  int key_bits = 1;   // the keys are below M^3: no sort passes over bits that are always zero
+  while (key_bits < 32 && ((size_t)1 << key_bits) < ncell) ++key_bits;
   if (M > 0)
     GBI_CHECK(cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, (const unsigned int*)nullptr, (unsigned int*)nullptr,
-                                              (const int*)nullptr, (int*)nullptr, N, 0, 32, ctx->stream));
+                                              (const int*)nullptr, (int*)nullptr, N, 0, key_bits, ctx->stream));
   const size_t K3 = (size_t)K * K * K;
   using C = typename Cplx<G>::t;
   using Q = typename Cplx<G>::q;
@@ -1111,7 +1150,7 @@ gbi_status run_periodic(gbi_ctx* ctx, int N, double L, double a, double eta, con
   // are the staging points and the two complex grids A, B
   const long long slots = std::max(nk, (long long)K);
   const size_t mesh_bytes = K > 0 ? K3 * (sizeof(Q) + 2 * sizeof(C)) : 0;
-  const PerBufs o = per_layout<T>(N, slots, ncell, sort_bytes, mesh_bytes);
+  const PerBufs o = per_layout<T>(N, slots, ncell, sort_bytes, mesh_bytes, M > 0);
   GBI_TRY(ensure(ctx, ctx->perbuf, o.total));
   char* b = static_cast<char*>(ctx->perbuf.p);
   T* pos = reinterpret_cast<T*>(b + o.o_pos);
@@ -1125,22 +1164,24 @@ gbi_status run_periodic(gbi_ctx* ctx, int N, double L, double a, double eta, con
   int* sidx = reinterpret_cast<int*>(b + o.o_sidx);
   int* cs = reinterpret_cast<int*>(b + o.o_cs);
   int* ce = reinterpret_cast<int*>(b + o.o_ce);
+  double* frac = reinterpret_cast<double*>(b + o.o_frac);
+  PmePoint<T>* pt = reinterpret_cast<PmePoint<T>*>(b + o.o_pt);
   if (nk > 0) {
     GBI_CHECK(cudaMemcpyAsync(kvd, kv.data(), sizeof(T) * kv.size(), cudaMemcpyHostToDevice, ctx->stream));
   }
   // records in cell order (M >= 3) or in input order (every pair)
   const int* order = nullptr;
   if (M > 0) {
-    k_per_keys<<<grid1(N), 256, 0, ctx->stream>>>(N, L, M, R, key, idx);
+    k_per_keys<<<grid1(N), 256, 0, ctx->stream>>>(N, L, M, R, key, idx, frac);
     size_t tb = sort_bytes;
-    GBI_CHECK(cub::DeviceRadixSort::SortPairs(b + o.o_tmp, tb, key, skey, idx, sidx, N, 0, 32, ctx->stream));
+    GBI_CHECK(cub::DeviceRadixSort::SortPairs(b + o.o_tmp, tb, key, skey, idx, sidx, N, 0, key_bits, ctx->stream));
     GBI_CHECK(cudaMemsetAsync(cs, 0, sizeof(int) * ncell, ctx->stream));
     GBI_CHECK(cudaMemsetAsync(ce, 0, sizeof(int) * ncell, ctx->stream));
     k_per_cell_bounds<<<grid1(N), 256, 0, ctx->stream>>>(N, skey, cs, ce);
     ctx->launches += 2;
     order = sidx;
   }
-  k_per_records<T><<<grid1(N), 256, 0, ctx->stream>>>(N, L, R, Fe, order, pos, frc);
+  k_per_records<T><<<grid1(N), 256, 0, ctx->stream>>>(N, L, R, M > 0 ? frac : nullptr, Fe, order, pos, frc, K, pt);
   if (M > 0) {
     // slices per cell: enough blocks for a cell of mean + 4 sigma records
     const double mean = double(N) / double(ncell);
@@ -1179,25 +1220,23 @@ gbi_status run_periodic(gbi_ctx* ctx, int N, double L, double a, double eta, con
     GBI_CHECK(cudaMemcpyAsync(twd, twh.data(), sizeof(G) * 2 * K, cudaMemcpyHostToDevice, ctx->stream));
     GBI_CHECK(cudaMemsetAsync(Qs, 0, sizeof(Q) * K3, ctx->stream));
     const unsigned lane_blocks = (unsigned)(((size_t)N * kPmeLanes + 127) / 128);
-    k_pme_spread<G><<<lane_blocks, 128, 0, ctx->stream>>>(N, K, R, L, Fe, sidx, Qs);
-    const int LB = pme_lines_per_block(K, sizeof(C));
-    int logLB = 0;
-    while ((1 << logLB) < LB) ++logLB;
+    k_pme_spread<G><<<lane_blocks, 128, 0, ctx->stream>>>(N, K, pt, frc, Qs);
+    const int LB = pme_lines<G>(K);
     const dim3 lines((unsigned)((size_t)K * K / LB), 2);
     const size_t fsm = sizeof(C) * ((size_t)LB * pme_row(K) + K);
-    // forward along z (from the staging points) and y, then x with the products and x back,
-    // then y and z back
-    const int logP = logLB - 2;   // 4 P rows = LB rows in shared memory
-    const unsigned xblocks = (unsigned)((size_t)K * K >> logP);
+    // forward along z (from the staging points) and y, then x with the products and x back
+    // (LB rows hold those of LB / 4 slots), then y and z back
+    const unsigned xblocks = (unsigned)((size_t)K * K * 4 / LB);
+    const G ks = G(2.0 * kPi / L), kc = G(8.0 * kPi / (L * L * L)), kq = G(0.25 / (p.xi * p.xi));
     cudaError_t e = cudaSuccess;
     switch (K / 16) {
 #define GBI_PME_FFT(N2)                                                                                     \
   case N2:                                                                                                  \
-    k_pme_fft4<G, N2><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, Qs, logLB, 2, 0, twd);                \
-    k_pme_fft4<G, N2><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, nullptr, logLB, 1, 0, twd);           \
-    k_pme_xconv<G, N2><<<xblocks, kPmeFftThreads, fsm, ctx->stream>>>(A, B, logP, L, p.xi, bmd, twd);       \
-    k_pme_fft4<G, N2><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, nullptr, logLB, 1, 1, twd);           \
-    k_pme_fft4<G, N2><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, nullptr, logLB, 2, 1, twd);           \
+    k_pme_fft4<G, N2, 2, false, true><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, Qs, twd);             \
+    k_pme_fft4<G, N2, 1, false, false><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, nullptr, twd);       \
+    k_pme_xconv<G, N2><<<xblocks, kPmeFftThreads, fsm, ctx->stream>>>(A, B, ks, kc, kq, bmd, twd);          \
+    k_pme_fft4<G, N2, 1, true, false><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, nullptr, twd);        \
+    k_pme_fft4<G, N2, 2, true, false><<<lines, kPmeFftThreads, fsm, ctx->stream>>>(A, nullptr, twd);        \
     break;
       GBI_PME_FFT(1)
       GBI_PME_FFT(2)
@@ -1209,7 +1248,9 @@ gbi_status run_periodic(gbi_ctx* ctx, int N, double L, double a, double eta, con
       default: e = cudaErrorInvalidValue;
     }
     GBI_CHECK(e);
-    k_pme_gather<G, T><<<lane_blocks, 128, 0, ctx->stream>>>(N, K, R, L, Fe, sidx, A, B, p.xi, a, eta, ur, Va, V);
+    k_pme_gather<G, T><<<lane_blocks, 128, 0, ctx->stream>>>(N, K, pt, Fe, sidx, A, B, 8.0 * p.xi / kSqrtPi,
+                                                            1.0 / (6.0 * kPi * eta * a), 1.0 / (8.0 * kPi * eta),
+                                                            ur, Va, V);
     ctx->launches += 7;
   }
   GBI_CHECK(cudaGetLastError());
