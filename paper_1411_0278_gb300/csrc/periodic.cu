@@ -312,7 +312,7 @@ __device__ __forceinline__ void per_real_staged(const T* pn, const T* sp, const 
 // per load), then only those are evaluated, so the lanes of a warp diverge only in how many of
 // 128 -- of 32 at a time the longest lane had twice the mean.  The four quarters' compensated sums
 // are added at the end.  Instruction issue bounds it: 15 % of the candidates are inside, a test
-// takes about 7 instructions and a term about 90.  N = 10^5: kRealUs.
+// takes about 7 instructions and a term about 90.  N = 10^5 (M = 12): 399 us, 550 before.
 constexpr int kPerCellThreads = 256;
 constexpr int kPerCellSlots = 64;
 constexpr int kPerCellQuarters = kPerCellThreads / kPerCellSlots;
@@ -852,7 +852,7 @@ __device__ __forceinline__ void pme_fft4_rows(typename Cplx<G>::t* sx, const typ
 // lines are read from the staging points instead (A = x + i y, B = z).  tw[t] = e^{-2 pi i t / K},
 // t < K.  Indices are 32-bit (K^3 <= 2^27).  Axis, direction and lines are template parameters:
 // with them as arguments two thirds of the ~106 instructions per element were index arithmetic
-// (ncu: issue 63 % active, FMA pipe 21 %).  K = 256: kFftUs a pass.
+// (ncu: issue 63 % active, FMA pipe 21 %).  K = 256: 109-123 us a pass (153 before), 0.65-0.73 of the copy bandwidth.
 template <typename G, int N2, int AXIS, bool INV, bool SRC>
 __global__ void __launch_bounds__(kPmeFftThreads, (sizeof(G) == 4 && N2 >= 16) ? 3 : 1)
     k_pme_fft4(typename Cplx<G>::t* __restrict__ grids, const typename Cplx<G>::q* __restrict__ src,
