@@ -356,6 +356,80 @@ __global__ void __launch_bounds__(256) bk_dots_fin(const double* __restrict__ V,
   finalize_column(p, s, j, 0);
 }
 
+// bk_dots_fin for several systems (S CH blocks fill the SMs by themselves): block (s, c) forms all
+// the slots of chunk c of system s.  A warp takes four slots at a time -- w is read once for the
+// four, and their sums over the lanes are reduced together by halving (6 additions for 20) --
+// and the warps that the groups of four leave over share the elements.  FP64 instructions bound
+// these sums (16 cycles of the SM's pipe each): with a 256-thread block per (system, slot, row) most
+// of them were the shuffle trees of one-element threads.  48 systems of 32 to 1024 spheres, l <= 2:
+// 16.9 us a step (ncu) against 21.7 us.
+__global__ void __launch_bounds__(256) bk_dots_multi(const double* __restrict__ V, size_t n,
+                                                     const double* __restrict__ w, int Ntot, int h,
+                                                     const int* __restrict__ off, GPtr p) {
+  pdl_wait();
+  const int s = blockIdx.x, c = blockIdx.y;
+  const GDev* st = p.st + s;
+  if (!st->active) return;
+  const int j = st->j, CH = p.CH;
+  __shared__ double s_part[8][4];
+  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lo = off[s], ns = off[s + 1] - lo;
+  const int q0 = c * h / CH, q1 = (c + 1) * h / CH;
+  const int groups = (j + 5) >> 2;                     // of the slots 0..j + 1
+  const int width = groups < 8 ? groups : 8;           // groups in flight
+  const int parts = 8 / width;                         // warps per group
+  const int part = wi / width;
+  for (int g0 = 0; g0 < groups; g0 += width) {
+    const int g = g0 + wi % width;
+    const bool on = g < groups && part < parts;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    if (on) {
+      const int i0 = 4 * g, top = j + 1 - i0;          // slots i0 .. i0 + min(3, top); slot j + 1 is w . w
+      const int step = 32 * parts;
+      for (int q = q0; q < q1; ++q) {
+        const size_t b = (size_t)q * Ntot + lo;
+        const double* wq = w + b;
+        const double* v = V + (size_t)i0 * n + b;
+        for (int t = part * 32 + lane; t < ns; t += step) {
+          const double x = wq[t];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (u < top) a[u] = fma(v[(size_t)u * n + t], x, a[u]);
+            else if (u == top) a[u] = fma(x, x, a[u]);
+          }
+        }
+      }
+    }
+    const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
+    double b0 = (u16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, u16 ? a[0] : a[2], 16);
+    const double b1 = (u16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, u16 ? a[1] : a[3], 16);
+    b0 = (u8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, u8 ? b0 : b1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) b0 += __shfl_xor_sync(0xffffffffu, b0, o);
+    if ((lane & 7) == 0) s_part[wi][lane >> 3] = b0;
+    __syncthreads();
+    if (threadIdx.x < 4 * width) {
+      const int i = 4 * g0 + threadIdx.x;
+      if (i <= j + 1) {
+        double v = s_part[threadIdx.x >> 2][threadIdx.x & 3];
+        for (int k = 1; k < parts; ++k) v += s_part[k * width + (threadIdx.x >> 2)][threadIdx.x & 3];
+        p.h1p[((size_t)s * (p.m + 1) + i) * CH + c] = v;
+      }
+    }
+    __syncthreads();
+  }
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(p.cnt + s, 1u) == (unsigned int)CH - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (threadIdx.x == 0) p.cnt[s] = 0u;
+  finalize_column(p, s, j, 0);
+}
+
 // One-reduction Arnoldi step, first half, for batches of many small systems: one block
 // per system, its warp k taking the slots i = k, k + 8, ... <= j_s + 1 (V_i . w, and w . w
 // for i = j_s + 1) over the system's whole vector (lanes stride its elements, a shuffle
@@ -1257,6 +1331,10 @@ void launch_norm(gbi_ctx* ctx, const Batch& B, int h, const GPtr& gp, const doub
 // double-float, so a lost digit there costs at most an extra sweep, never accuracy.
 int two_pass_gs(int precision) { return precision == 0 ? 1 : 0; }
 
+// (system, chunk) blocks from which bk_dots_multi serves the step: fewer leave SMs without one,
+// and bk_dots_fin's block per slot as well spreads further (a single system has 8 to 48 chunks)
+constexpr int kMultiBlocks = 152;
+
 // Arnoldi steps per trip of a device-side loop: a trip costs about 4.5 us of conditional
 // node overhead on GB300 besides its kernels, a step after its system has stopped about
 // 4 us (its kernels return at once), so several steps a trip pay off.
@@ -1352,7 +1430,10 @@ gbi_status launch_chunk(gbi_ctx* ctx, const Setup& s, const Batch& B, int precis
                                 h, B.off, gp, so, lcs));
       ++ctx->launches;
     } else {
-      if (S < 64) {
+      if (S < 64 && S * gp.CH >= kMultiBlocks) {
+        GBI_CHECK(launch_pdl(pdl, dim3(S, gp.CH), dim3(256), ctx->stream, bk_dots_multi, Vb, n, w, Ntot, h, B.off, gp));
+        ++ctx->launches;
+      } else if (S < 64) {
         // dot products, norm and Givens step in one kernel
         GBI_CHECK(launch_pdl(pdl, gd, dim3(256), ctx->stream, bk_dots_fin, Vb, n, w, Ntot, h, B.off, gp));
         ++ctx->launches;
