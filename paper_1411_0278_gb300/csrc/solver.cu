@@ -3,6 +3,7 @@
 // tests in kernels, the Arnoldi steps of a cycle replayed from a CUDA graph with a
 // device-side WHILE loop, and the solve sequence (right-hand side, refinement sweeps,
 // output pass).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -735,6 +736,148 @@ __global__ void __launch_bounds__(256) bk_step_fused(double* V, size_t n, double
   }
 }
 
+// The whole orthogonalisation of one system of up to kClusterElems vector elements: one
+// cluster of eight blocks, each owning a slice of the vectors (w in its shared memory), with the
+// partial sums exchanged through distributed shared memory and every block adding them in rank
+// order.  two_pass: both Gram-Schmidt rounds and the norm of the result (three cluster
+// barriers), otherwise one round and the norm from |w|^2 - sum c_i^2 (one).  Block 0 runs the
+// Givens step and, in the graphs, ends the step.  Small systems are bound by the launches and
+// serial chains of a step: 64 spheres at l <= 2 in FP64 took seven kernels after the pair pass
+// (22.7 us as bk_step_fused with its grid barriers), this one 12 (ncu).  Beyond the limits below the
+// eight SMs' FP64 pipes cost more than the launches saved.  Whole solves, separate kernels -> this
+// one: two rounds n = 512: 584 -> 481 us, 4096: 1683 -> 1648, 6144: 3393 -> 3416; one round n = 512: 402 ->
+// 381, 1536: 421 -> 413, 3072: 483 -> 517.
+constexpr int kClusterBlocks = 8, kClusterThreads = 256;
+constexpr int kClusterElems = 4096, kClusterElemsOne = 1536;   // two Gram-Schmidt rounds, one
+constexpr int kClusterSlice = kClusterElems / kClusterBlocks;
+
+__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kClusterThreads)
+    bk_step_cluster(double* __restrict__ V, size_t n, const double* __restrict__ w, int Ntot, int h, GPtr p, SrcOut so,
+                    int two_pass, LoopCtl lc) {
+  namespace cg = cooperative_groups;
+  __shared__ double s_w[kClusterSlice];
+  __shared__ double s_p[2][kGmMaxM + 4], s_c[kGmMaxM + 4], s_c2[kGmMaxM + 4], s_cs[kGmMaxM], s_sn[kGmMaxM], s_red[8];
+  __shared__ double s_hn, s_ihn;
+  pdl_wait();
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  GDev* st = p.st;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (!st->active) {   // the same decision in every block: block 0 writes the state after the barriers
+    if (lc.on && rank == 0 && tid == 0) {
+      *lc.nact = 0;
+      if (lc.on == 2) {
+        if (lc.steps != nullptr) *lc.steps += 1;
+        cudaGraphSetConditional(lc.h, 0u);
+      }
+    }
+    return;
+  }
+  const int j = st->j, m = p.m;
+  const int slice = (int)((n + kClusterBlocks - 1) / kClusterBlocks);
+  const int t0 = rank * slice, len = max(0, min((int)n - t0, slice));
+  for (int t = tid; t < len; t += kClusterThreads) s_w[t] = w[t0 + t];
+  __syncthreads();
+  const double* Vs = V + t0;
+  // out[i] = V_i . w over the slice for i <= j, and w . w in slot j + 1 if top > j: four slots per
+  // warp at a time, reduced together
+  auto dots = [&](double* out, int top) {
+    for (int i0 = 4 * warp; i0 <= top; i0 += 32) {
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int t = lane; t < len; t += 32) {
+        const double x = s_w[t];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u;
+          if (i <= j) a[u] = fma(Vs[(size_t)i * n + t], x, a[u]);
+          else if (i == top) a[u] = fma(x, x, a[u]);
+        }
+      }
+      const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
+      double b0 = (u16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, u16 ? a[0] : a[2], 16);
+      const double b1 = (u16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, u16 ? a[1] : a[3], 16);
+      b0 = (u8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, u8 ? b0 : b1, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) b0 += __shfl_xor_sync(0xffffffffu, b0, o);
+      const int i = i0 + (lane >> 3);
+      if ((lane & 7) == 0 && i <= top) out[i] = b0;
+    }
+  };
+  // out[i] = the sum of every block's in[i], in rank order
+  auto gather = [&](double* in, double* out, int top) {
+    for (int i = tid; i <= top; i += kClusterThreads) {
+      double q[kClusterBlocks];
+#pragma unroll
+      for (int r = 0; r < kClusterBlocks; ++r) q[r] = cl.map_shared_rank(in, r)[i];
+      double c = q[0];
+#pragma unroll
+      for (int r = 1; r < kClusterBlocks; ++r) c += q[r];
+      out[i] = c;
+    }
+    __syncthreads();
+  };
+  auto subtract = [&](const double* c) {
+    for (int t = tid; t < len; t += kClusterThreads) {
+      double a = s_w[t];
+#pragma unroll 4
+      for (int i = 0; i <= j; ++i) a = fma(-c[i], Vs[(size_t)i * n + t], a);
+      s_w[t] = a;
+    }
+    __syncthreads();
+  };
+  dots(s_p[0], two_pass ? j : j + 1);
+  cl.sync();
+  gather(s_p[0], s_c, two_pass ? j : j + 1);
+  subtract(s_c);
+  if (two_pass) {
+    dots(s_p[1], j);
+    cl.sync();
+    gather(s_p[1], s_c2, j);
+    subtract(s_c2);
+    double a = 0.0;
+    for (int t = tid; t < len; t += kClusterThreads) a = fma(s_w[t], s_w[t], a);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) s_red[warp] = a;
+    __syncthreads();
+    if (tid == 0) {
+      double v = s_red[0];
+      for (int k = 1; k < 8; ++k) v += s_red[k];
+      s_p[0][kGmMaxM + 3] = v;   // no block reads slot kGmMaxM + 3 of the first round
+    }
+    cl.sync();
+    if (tid == 0) {
+      double nrm = 0.0;
+      for (int r = 0; r < kClusterBlocks; ++r) nrm += cl.map_shared_rank(s_p[0], r)[kGmMaxM + 3];
+      root_and_inverse(nrm, s_hn, s_ihn);
+    }
+    for (int i = tid; i <= j; i += kClusterThreads) s_c[i] += s_c2[i];
+  } else if (tid == 0) {
+    double nrm = s_c[j + 1];
+    for (int i = 0; i <= j; ++i) nrm = fma(-s_c[i], s_c[i], nrm);
+    root_and_inverse(nrm, s_hn, s_ihn);
+  }
+  __syncthreads();
+  const double hn = s_hn, inv = hn > 1e-300 ? s_ihn : 0.0;
+  for (int t = tid; t < len; t += kClusterThreads) {
+    const double v = s_w[t] * inv;
+    const int e = t0 + t, q = e / Ntot;
+    V[(size_t)(j + 1) * n + e] = v;
+    write_src(so, Ntot, h, q, e - q * Ntot, v);
+  }
+  if (rank == 0) {
+    givens_step(p, 0, j, hn, s_ihn, s_c, s_cs, s_sn);
+    if (lc.on && tid == 0) {
+      *lc.nact = 0;
+      if (lc.on == 2) {
+        if (lc.steps != nullptr) *lc.steps += 1;
+        cudaGraphSetConditional(lc.h, st->active ? 1u : 0u);
+      }
+    }
+  }
+  cl.sync();   // no block leaves while another may read its shared memory
+}
+
 // The whole orthogonalisation of the one-reduction step for batches of small systems
 // (warp_systems): one warp per system, kStepWarps systems per block, against one block per
 // system for the dot products and the Givens step and a second kernel for the vectors.  GB300's
@@ -1395,6 +1538,13 @@ gbi_status launch_chunk(gbi_ctx* ctx, const Setup& s, const Batch& B, int precis
     if (lc.on) lcs.on = c + 1 < kChunk ? 1 : 2;
     pa.pdl = pdl && c > 0;
     GBI_CHECK(run_pairs(ctx, s.trunc, SET_H, SET_H, precision, pa));
+    if (S == 1 && n <= (size_t)(two ? kClusterElems : kClusterElemsOne)) {
+      // one small system: the orthogonalisation on one cluster
+      GBI_CHECK(launch_pdl(pdl, dim3(kClusterBlocks), dim3(kClusterThreads), ctx->stream, bk_step_cluster, Vb, n, w,
+                           Ntot, h, gp, so, two, lcs));
+      ++ctx->launches;
+      continue;
+    }
     if (fused && S == 1) {
       // a single system launched step by step: the whole orthogonalisation in one kernel.
       // Its grid barriers need every block resident at once: a cooperative launch
