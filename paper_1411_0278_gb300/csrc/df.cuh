@@ -66,15 +66,56 @@ __host__ __device__ __forceinline__ df& operator+=(df& a, df b) {
   return a;
 }
 
-// a * b + c: the product's rounding error terms are folded into the sum (12 FP32
-// operations instead of 15 for a separate * and +)
+// a product that the compiler must not fuse into a later sum
+__host__ __device__ __forceinline__ float df_rmul(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+
+// a * b + c in 10 FP32 operations.  With p = fl(a.hi b.hi), s = fl(p + c.hi) and Knuth's split
+// v = s - p, w = s - v of the sum, both c.hi - v and p - w are exact and add up to p + c.hi - s; the
+// product's error a.hi b.hi - p rides on the second one in a single FMA, a.hi b.hi - w.  (A product with
+// its error followed by a two-sum takes 12.)  The double-float pair passes are bound by the FP32 pipe
+// (70% busy), so operations are their time: with this, df_mul and df_rsqrt an H/H pair of l <= 3 takes
+// 3360 instead of 4485 instructions, 148 us instead of 181 at N = 1024 (ncu), at a smaller error of the pair
+// block (rms 3.3e-14 of its norm, before 3.8e-14).
 __host__ __device__ __forceinline__ df df_fma(df a, df b, df c) {
-  const float p = a.hi * b.hi;
+  const float p = df_rmul(a.hi, b.hi);
+  const float s = p + c.hi;
+  const float v = s - p;
+  const float w = s - v;
+  float e = (c.hi - v) + c.lo;
+  e = fmaf(a.hi, b.lo, e);
+  e = fmaf(a.lo, b.hi, e);
+  return df(s, fmaf(a.hi, b.hi, -w) + e);
+}
+
+// a * b left unnormalised like the sums (4 operations, operator* 7): for factors and addends that are
+// used once or twice.  Powers, whose errors would build up, use operator* (unnormalised powers too: rms
+// 7.9e-14).
+__host__ __device__ __forceinline__ df df_mul(df a, df b) {
+  const float p = df_rmul(a.hi, b.hi);
   float e = fmaf(a.hi, b.hi, -p);
   e = fmaf(a.hi, b.lo, e);
   e = fmaf(a.lo, b.hi, e);
-  const df s = df_two_sum(p, c.hi);
-  return df(s.hi, s.lo + (e + c.lo));
+  return df(p, e);
+}
+
+// with a factor that is exact in FP32: no a.lo b.hi term
+__host__ __device__ __forceinline__ df df_fma(float a, df b, df c) {
+  const float p = df_rmul(a, b.hi);
+  const float s = p + c.hi;
+  const float v = s - p;
+  const float w = s - v;
+  const float e = fmaf(a, b.lo, (c.hi - v) + c.lo);
+  return df(s, fmaf(a, b.hi, -w) + e);
+}
+__host__ __device__ __forceinline__ df df_mul(float a, df b) {
+  const float p = df_rmul(a, b.hi);
+  return df(p, fmaf(a, b.lo, fmaf(a, b.hi, -p)));
 }
 
 __host__ __device__ __forceinline__ bool operator>(df a, df b) {
@@ -83,17 +124,21 @@ __host__ __device__ __forceinline__ bool operator>(df a, df b) {
 
 __host__ __device__ __forceinline__ double df_to_double(df a) { return double(a.hi) + double(a.lo); }
 
-// 1/sqrt(a): FP32 estimate, then one Newton step y + y (1 - a y^2) / 2 in double-float.
+// 1/sqrt(a): FP32 estimate y, residual r = 1 - a y^2 (one FMA each for the parts of a and y^2), then
+// y (1 + r/2 + 3 r^2/8).  r is some 2^-22, so FP32 carries the correction (11 operations; a Newton step in
+// double-float took 33 and left the r^2 term out).
 __host__ __device__ __forceinline__ df df_rsqrt(df a) {
 #ifdef __CUDA_ARCH__
   const float y = rsqrtf(a.hi);
 #else
   const float y = 1.0f / sqrtf(a.hi);
 #endif
-  const df yy = df_two_prod(y, y);
-  const df r = df(1.0f, 0.0f) - a * yy;
-  const df hy = df(0.5f * y, 0.0f);
-  return df(y, 0.0f) + hy * r;
+  const float q = df_rmul(y, y);
+  const float ql = fmaf(y, y, -q);
+  float r = fmaf(-a.hi, q, 1.0f);
+  r = fmaf(-a.hi, ql, r);
+  r = fmaf(-a.lo, q, r);
+  return df_fast_two_sum(y, y * (r * fmaf(0.375f, r, 0.5f)));
 }
 
 #ifdef __CUDACC__
@@ -105,7 +150,16 @@ __device__ __forceinline__ df df_shfl_xor(df v, int o) {
 }  // namespace gbi
 
 // a * b + c in the arithmetic of T (fused where the type has a fused form); the
-// generated pair-frame code chains its sums of products through this
+// generated pair-frame code chains its sums of products through this.  A float first factor is a
+// constant that is exact in FP32.
 __host__ __device__ __forceinline__ float gbi_fmac(float a, float b, float c) { return fmaf(a, b, c); }
 __host__ __device__ __forceinline__ double gbi_fmac(double a, double b, double c) { return fma(a, b, c); }
+__host__ __device__ __forceinline__ double gbi_fmac(float a, double b, double c) { return fma(double(a), b, c); }
 __host__ __device__ __forceinline__ gbi::df gbi_fmac(gbi::df a, gbi::df b, gbi::df c) { return gbi::df_fma(a, b, c); }
+__host__ __device__ __forceinline__ gbi::df gbi_fmac(float a, gbi::df b, gbi::df c) { return gbi::df_fma(a, b, c); }
+// a * b that is added up or used as a factor once or twice
+__host__ __device__ __forceinline__ float gbi_mul(float a, float b) { return a * b; }
+__host__ __device__ __forceinline__ double gbi_mul(double a, double b) { return a * b; }
+__host__ __device__ __forceinline__ double gbi_mul(float a, double b) { return double(a) * b; }
+__host__ __device__ __forceinline__ gbi::df gbi_mul(gbi::df a, gbi::df b) { return gbi::df_mul(a, b); }
+__host__ __device__ __forceinline__ gbi::df gbi_mul(float a, gbi::df b) { return gbi::df_mul(a, b); }

@@ -92,7 +92,7 @@ __host__ __device__ __forceinline__ void dapplyT(const DMats<T>& dm, const T* in
 template <int J, typename T>
 __host__ __device__ __forceinline__ T eps_pow(const T* ep, T v) {
   if constexpr (J == 0) return v;
-  else return ep[J] * v;
+  else return gbi_mul(ep[J], v);
 }
 
 // Rotate the column modes [M, MEND) of x (absolute component index) into the pair
@@ -112,8 +112,8 @@ __host__ __device__ __forceinline__ void to_pair_frame(const T* x, T* xs, const 
     for (int mm = 1; mm <= k; ++mm) {
       const T c = eps_pow<l>(ep, cm[mm]), s = eps_pow<l>(ep, sm[mm]);
       const T xp = x[o + k + mm], xn = x[o + k - mm];
-      t[k + mm] = gbi_fmac(c, xp, s * xn);
-      t[k - mm] = gbi_fmac(c, xn, -(s * xp));
+      t[k + mm] = gbi_fmac(c, xp, gbi_mul(s, xn));
+      t[k - mm] = gbi_fmac(c, xn, -gbi_mul(s, xp));
     }
     dapply<k, T>(dm, t, xs + o);
     to_pair_frame<TR, T, M + 1, MEND>(x, xs, cm, sm, dm, ep);
@@ -135,7 +135,7 @@ __host__ __device__ __forceinline__ void from_pair_frame(const T* yy, T* acc, co
     acc[o - R0 + k] = gbi_fmac(ep[l + 1], t[k], acc[o - R0 + k]);
 #pragma unroll
     for (int mm = 1; mm <= k; ++mm) {
-      const T c = ep[l + 1] * cm[mm], s = ep[l + 1] * sm[mm];
+      const T c = gbi_mul(ep[l + 1], cm[mm]), s = gbi_mul(ep[l + 1], sm[mm]);
       const T tp = t[k + mm], tn = t[k - mm];
       acc[o - R0 + k + mm] = gbi_fmac(c, tp, gbi_fmac(-s, tn, acc[o - R0 + k + mm]));
       acc[o - R0 + k - mm] = gbi_fmac(s, tp, gbi_fmac(c, tn, acc[o - R0 + k - mm]));
@@ -186,6 +186,18 @@ template <int TR, int ROWS, int COLS> struct PassShape {
   static constexpr int MAXK = MAXK_R > MAXK_C ? MAXK_R : MAXK_C;
 };
 
+// |rho|^2 and its part in the xy plane
+template <typename T>
+__host__ __device__ __forceinline__ T pair_r2(T dx, T dy, T dz, T& rxy2) {
+  if constexpr (std::is_same<T, df>::value) {
+    rxy2 = df_fma(dx, dx, df_mul(dy, dy));
+    return df_fma(dz, dz, rxy2);
+  } else {
+    rxy2 = dx * dx + dy * dy;
+    return rxy2 + dz * dz;
+  }
+}
+
 // One ordered pair: acc[p - R0] += sum_q C-rotated block [p][q] * xl[q] for
 // rho = (dx, dy, dz) = R_n - R_m, xl indexed by absolute component (columns only).
 // The 1/a factor of the block is applied by the caller.
@@ -193,8 +205,8 @@ template <int TR, int ROWS, int COLS, typename T>
 __host__ __device__ __forceinline__ void pair_body(T dx, T dy, T dz, T a, const T* xl, T* acc) {
   using S = PassShape<TR, ROWS, COLS>;
   constexpr int MAXK = S::MAXK;
-  const T rxy2 = dx * dx + dy * dy;
-  const T r2 = rxy2 + dz * dz;
+  T rxy2;
+  const T r2 = pair_r2(dx, dy, dz, rxy2);
   const T rinv = gbi_rsqrt(r2);
   const T eps = a * rinv;
   const T e2 = eps * eps;
@@ -212,8 +224,8 @@ __host__ __device__ __forceinline__ void pair_body(T dx, T dy, T dz, T a, const 
   cm[1] = cphi; sm[1] = sphi;
 #pragma unroll
   for (int mm = 2; mm <= MAXK; ++mm) {
-    cm[mm] = gbi_fmac(cm[mm - 1], cphi, -(sm[mm - 1] * sphi));
-    sm[mm] = gbi_fmac(sm[mm - 1], cphi, cm[mm - 1] * sphi);
+    cm[mm] = gbi_fmac(cm[mm - 1], cphi, -gbi_mul(sm[mm - 1], sphi));
+    sm[mm] = gbi_fmac(sm[mm - 1], cphi, gbi_mul(cm[mm - 1], sphi));
   }
   // rotation about y by -theta: cos = ct, sin = -st
   DMats<T> dm;
@@ -451,7 +463,8 @@ __device__ __forceinline__ void stream_source(const PairArgs& args, const float4
     dy = (th.y - sh.y) + (tl.y - sl.y);
     dz = (th.z - sh.z) + (tl.z - sl.z);
   }
-  min_r2 = fminf(min_r2, float(dx * dx + dy * dy + dz * dz));
+  T rxy2;
+  min_r2 = fminf(min_r2, float(pair_r2(dx, dy, dz, rxy2)));   // shared with pair_body's
   T xl[D];
 #pragma unroll
   for (int q = 0; q < NC; ++q) {

@@ -148,7 +148,8 @@ __device__ __forceinline__ void tile_source(const float4* __restrict__ srec, con
     dy = (th.y - sh.y) + (tl.y - sl.y);
     dz = (th.z - sh.z) + (tl.z - sl.z);
   }
-  min_r2 = fminf(min_r2, float(dx * dx + dy * dy + dz * dz));
+  T rxy2;
+  min_r2 = fminf(min_r2, float(pair_r2(dx, dy, dz, rxy2)));   // shared with pair_body's
   T xl[D];
 #pragma unroll
   for (int q = 0; q < NC; ++q) {

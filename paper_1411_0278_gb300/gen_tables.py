@@ -21,6 +21,7 @@ script runs on both build machines and its output is deterministic.
 """
 import math
 import os
+import struct
 import sys
 from fractions import Fraction as Fr
 
@@ -416,15 +417,30 @@ def fmt(v):
     return repr(float(v))
 
 
+def factor(a):
+    """A constant factor "T(c)" that is exact in FP32 as a float literal (one operation less in
+    double-float); any other factor as it is."""
+    if a.startswith("T("):
+        c = float(a[2:-1])
+        if struct.unpack("f", struct.pack("f", c))[0] == c:
+            return repr(c) + "f"
+    return a
+
+
 def fma_chain(terms):
     """C++ expression for the sum of products [(a, b), ...] as a chain of gbi_fmac calls:
     the first product is a plain multiply, every later one is fused into the sum."""
     if not terms:
         return "T(0)"
     a0, b0 = terms[0]
-    expr = a0 if b0 is None else "%s * %s" % (a0, b0)
+    if b0 is None:
+        expr = a0
+    elif a0 in ("T(1.0)", "T(-1.0)"):
+        expr = b0 if a0 == "T(1.0)" else "(-%s)" % b0
+    else:
+        expr = "gbi_mul(%s, %s)" % (factor(a0), b0)
     for a, b in terms[1:]:
-        expr = "(%s + %s)" % (expr, a) if b is None else "gbi_fmac(%s, %s, %s)" % (a, b, expr)
+        expr = "(%s + %s)" % (expr, a) if b is None else "gbi_fmac(%s, %s, %s)" % (factor(a), b, expr)
     return expr
 
 
@@ -483,7 +499,8 @@ def emit(path):
                     rows.setdefault(mu, []).append((e, nu))
             for o in range(-k, k + 1):
                 terms = rows.get(o, [])
-                w("  out[%d] = %s;" % (o + k, fma_chain([("dm[%d]" % e, "in[%d]" % (i + k)) for e, i in terms])))
+                w("  out[%d] = %s;" % (o + k, fma_chain([("T(1.0)" if entries[e][1] == {(0, 0): 1} else "dm[%d]" % e,
+                                                             "in[%d]" % (i + k)) for e, i in terms])))
             w("}")
     w("")
     # packing helpers for the trap inputs: U_mu . v^2 (mu = -2..2) and the Cartesian
