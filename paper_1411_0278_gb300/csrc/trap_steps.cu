@@ -16,7 +16,7 @@
 // A step is two kernels: the pair sums, and one that adds the splits, moves the spheres and
 // writes the next step's source records (the general call sequence: six).  Up to kStepsSmall
 // spheres one block runs all the steps in one launch.  Microseconds a step, before -> now:
-// N = 2: 26.7 -> 2.1, 64: 45 -> 8.3, 128: 45 -> 9.7, 1000: 53 -> 21.5, 10^4: 348 -> 256 (pairs 310 -> 242).
+// N = 2: 26.7 -> 2.0, 64: 45 -> 9.1, 128: 45 -> 14.7, 1000: 53 -> 16.5, 10^4: 348 -> 256 (pairs 310 -> 242).
 #include <cuda_runtime.h>
 
 #include <type_traits>
@@ -139,13 +139,17 @@ __global__ void k_steps_records(const StepPar c, const double* __restrict__ R, c
   step_record<DIP>(c, R + 3 * (size_t)n, p + 3 * (size_t)n, rec + (size_t)n * StepRec<DIP>::W);
 }
 
-// Pair sums of the sources [blockIdx.y chunk, + chunk) for four targets per thread, two at a
+// Pair sums of the sources [blockIdx.y chunk, + chunk) for 2 kStepTG targets per thread, two at a
 // time in paired instructions; the tile's records sit in shared memory with every word doubled,
 // so that one 16-byte load gives two broadcast operands (as trap_pairs_f2).
-constexpr int kStepThreads = 128, kStepTG = 2, kStepTile = 128, kStepMinBlocks = 4;
+// (The sources are split and added up as in trap_kernel.cu, so the sums are the same bits.)  Up to
+// kStepsNarrow spheres, where that leaves a few blocks (N = 1000: 32), the block is one warp with two
+// targets per thread.
+constexpr int kStepTile = 128;
+constexpr int kStepsNarrow = 2048;
 
-template <bool DIP>
-__global__ void __launch_bounds__(kStepThreads, kStepMinBlocks)
+template <bool DIP, int kStepThreads, int kStepTG, int kMinBlocks>
+__global__ void __launch_bounds__(kStepThreads, kMinBlocks)
     k_steps_pairs(const StepPar c, const float* __restrict__ rec, int chunk, float* __restrict__ partial) {
   constexpr int W = StepRec<DIP>::W, TI = 2 * kStepTG;
   pdl_wait();
@@ -260,22 +264,28 @@ __global__ void __launch_bounds__(6 * kMoveSpheres)
 // All the steps of a small suspension in one block.  Four lanes per sphere hold its centre and
 // orientation, one component each (the fourth idles): an FP64 instruction takes the SM's pipe 16
 // cycles and its result 64, whatever the lanes, so the update and the next record are written
-// with the components side by side.  G lanes per target share its sources (FP32 sums per lane,
-// added over the lanes in FP64); two block barriers a step.  A step is bound by the latency of the
-// FP64 chain from the sums to the next record and, towards kStepsSmall spheres, by the pairs on
-// the one SM: 8.3 us at N = 64 and 11.3 at 96, where the two kernels' launches take 9.3.
+// with the components side by side.  A target's sources are summed one after the other, as in
+// trap_kernel.cu, so that orbits with close encounters, which amplify a last bit by ten thousand within
+// fifty steps, stay the same; V and Omega are summed by different threads.  (Several lanes per target added
+// in FP64 took 8.3 us at N = 64 and left R 8e-9 off.)  A step is bound by the latency of the pair sums and of the
+// FP64 chain from them to the next record: 2.0 us at N = 2, 4.8 at 32, 9.1 at 64, where the two
+// kernels take 14.
 constexpr int kSmallThreads = 512;
 constexpr int kStepsSmall = 72;
 
 template <bool DIP>
 __global__ void __launch_bounds__(kSmallThreads)
-    k_steps_small(const StepPar c, int nsteps, int G, double* __restrict__ R, double* __restrict__ p) {
+    k_steps_small(const StepPar c, int nsteps, int G, int chunk, int half, double* __restrict__ R,
+                  double* __restrict__ p) {
   constexpr int W = StepRec<DIP>::W;
   constexpr unsigned int kAll = 0xffffffffu;
   __shared__ __align__(16) float s_rec[kStepsSmall * W];
-  __shared__ double s_sum[kStepsSmall][6];
+  __shared__ float s_part[2][kStepsSmall][6];
   const int tid = threadIdx.x, N = c.N;
-  const int n = tid / G, sub = tid & (G - 1);
+  // the sums' threads: split `sub` of target n, the velocity in the first part of the block, the
+  // angular velocity in the second
+  const bool angular = tid >= half;
+  const int item = angular ? tid - half : tid, n = item / G, sub = item - n * G;
   const StepC<float> k(c.a);
   // the state's lanes: sphere tid / 4, component tid % 4
   const bool owner = (tid & ~31) < 4 * N;   // the whole warp takes part in the exchanges
@@ -306,7 +316,6 @@ __global__ void __launch_bounds__(kSmallThreads)
   }
   for (int step = 0; step < nsteps; ++step) {
     __syncthreads();
-    float v[3] = {0.f, 0.f, 0.f}, w[3] = {0.f, 0.f, 0.f};
     if (n < N) {
       float ph[3], pl[3];
 #pragma unroll
@@ -314,42 +323,48 @@ __global__ void __launch_bounds__(kSmallThreads)
         ph[q] = s_rec[n * W + q];
         pl[q] = s_rec[n * W + 3 + q];
       }
-      for (int m = sub; m < N; m += G) {
-        if (m == n) continue;
-        float q[W];
-        const float4* r4 = reinterpret_cast<const float4*>(s_rec + m * W);
+      const int m0 = sub * chunk, m1 = min(N, m0 + chunk);
+      // both sums of every source; the one that a thread does not keep drops out
+      auto sum = [&](float* v, float* w) {
+#pragma unroll 2
+        for (int m = m0; m < m1; ++m) {
+          float q[W];
+          const float4* r4 = reinterpret_cast<const float4*>(s_rec + m * W);
 #pragma unroll
-        for (int i = 0; i < W / 4; ++i) {
-          const float4 t = r4[i];
-          q[4 * i] = t.x;
-          q[4 * i + 1] = t.y;
-          q[4 * i + 2] = t.z;
-          q[4 * i + 3] = t.w;
+          for (int i = 0; i < W / 4; ++i) {
+            const float4 t = r4[i];
+            q[4 * i] = t.x;
+            q[4 * i + 1] = t.y;
+            q[4 * i + 2] = t.z;
+            q[4 * i + 3] = t.w;
+          }
+          step_pair<DIP>(q, ph, pl, k, v, w, [&](float& ri) {
+            if (m == n) ri = 0.f;
+          });
         }
-        step_pair<DIP>(q, ph, pl, k, v, w, [](float&) {});
+      };
+      float v[3] = {0.f, 0.f, 0.f}, w[3] = {0.f, 0.f, 0.f};
+      float* o = s_part[sub][n] + (angular ? 3 : 0);
+      if (angular) {
+        sum(v, w);
+        o[0] = w[0], o[1] = w[1], o[2] = w[2];
+      } else {
+        sum(v, w);
+        o[0] = v[0], o[1] = v[1], o[2] = v[2];
       }
-    }
-    double s[6];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      s[q] = double(v[q]);
-      s[3 + q] = double(w[q]);
-    }
-    for (int o = G >> 1; o > 0; o >>= 1) {
-#pragma unroll
-      for (int q = 0; q < 6; ++q) s[q] += __shfl_xor_sync(kAll, s[q], o);
-    }
-    if (n < N && sub == 0) {
-#pragma unroll
-      for (int q = 0; q < 6; ++q) s_sum[n][q] = s[q];
     }
     __syncthreads();
     if (owner) {
       // step_move, a component per lane
-      const double* sm = s_sum[on];
+      // (the splits' sums in order)
+      auto total = [&](int q) {
+        double t = double(s_part[0][on][q]);
+        if (G > 1) t += double(s_part[1][on][q]);
+        return t;
+      };
       const double p1 = __shfl_sync(kAll, pc, l1), p2 = __shfl_sync(kAll, pc, l2);
-      Rc += c.dt * (c.vs * pc + c.mt * (-c.k * Rc) + sm[oc]);
-      const double q = pc + c.dt * (sm[3 + c1] * p2 - sm[3 + c2] * p1);
+      Rc += c.dt * (c.vs * pc + c.mt * (-c.k * Rc) + total(oc));
+      const double q = pc + c.dt * (total(3 + c1) * p2 - total(3 + c2) * p1);
       const double sq = q * q;
       const double s0 = __shfl_sync(kAll, sq, l0), s1 = __shfl_sync(kAll, sq, l0 + 1), s2 = __shfl_sync(kAll, sq, l0 + 2);
       pc = q * rsqrt(s0 + s1 + s2);
@@ -362,39 +377,26 @@ __global__ void __launch_bounds__(kSmallThreads)
   }
 }
 
-// Splits of the sources: as many as keep every target block's splits within one wave of the
-// resident blocks, at least 64 sources each, or 16 up to 2048 spheres, where 64 would leave most
-// SMs idle (N = 1000: 32 blocks).
-int steps_splits(int N, int sms) {
-  const int tb = (N + kStepThreads * 2 * kStepTG - 1) / (kStepThreads * 2 * kStepTG);
-  int s = sms * kStepMinBlocks / tb;
-  const int most = N <= 2048 ? (N + 15) / 16 : (N + 63) / 64;
-  if (s > most) s = most;
-  return s < 1 ? 1 : s;
-}
-
 template <bool DIP>
 gbi_status run_steps(gbi_ctx* ctx, const StepPar& c, int nsteps, double* R, double* p) {
   constexpr int W = StepRec<DIP>::W;
   const double flops = trap_flops() * double(c.N) * double(c.N - 1);
+  const int ns = trap_splits(c.N, 1), chunk = (c.N + ns - 1) / ns;   // at most 2 splits up to kStepsSmall
   if (c.N <= kStepsSmall && !ctx->prof) {
-    int G = 1;   // lanes per target: no more than there are sources
-    while (G < 32 && 2 * G <= c.N && 2 * G * c.N <= kSmallThreads) G <<= 1;
-    const int threads = (c.N * (G > 4 ? G : 4) + 31) / 32 * 32;   // at least four per sphere
+    const int half = (c.N * ns + 31) / 32 * 32;   // threads of one kind of sum
+    const int threads = half + half > 4 * c.N ? half + half : (4 * c.N + 31) / 32 * 32;
     // a launch stays below some ten milliseconds
     for (int done = 0; done < nsteps; done += 4096) {
-      k_steps_small<DIP><<<1, threads, 0, ctx->stream>>>(c, nsteps - done < 4096 ? nsteps - done : 4096, G, R, p);
+      k_steps_small<DIP><<<1, threads, 0, ctx->stream>>>(c, nsteps - done < 4096 ? nsteps - done : 4096, ns, chunk,
+                                                      half, R, p);
       ++ctx->launches;
     }
     GBI_CHECK(cudaGetLastError());
     return GBI_OK;
   }
-  const int ns = steps_splits(c.N, sm_count(ctx));
-  const int chunk = (c.N + ns - 1) / ns;
   GBI_TRY(ensure(ctx, ctx->trapbuf, sizeof(float) * ((size_t)c.N * W + (size_t)ns * c.N * 6)));
   float* rec = P<float>(ctx->trapbuf);
   float* partial = rec + (size_t)c.N * W;
-  const dim3 grid((c.N + kStepThreads * 2 * kStepTG - 1) / (kStepThreads * 2 * kStepTG), ns);
   const unsigned move = (unsigned)((c.N + kMoveSpheres - 1) / kMoveSpheres);
   k_steps_records<DIP><<<grid1(c.N, 128), 128, 0, ctx->stream>>>(c, R, p, rec);
   ++ctx->launches;
@@ -403,8 +405,11 @@ gbi_status run_steps(gbi_ctx* ctx, const StepPar& c, int nsteps, double* R, doub
   const float* cpart = partial;
   for (int s = 0; s < nsteps; ++s) {
     GBI_CHECK(timed(ctx, 28, flops, 1, [&] {
-      return launch_pdl(ctx->pdl && !ctx->prof, grid, dim3(kStepThreads), ctx->stream, k_steps_pairs<DIP>, c, crec,
-                        chunk, partial);
+      if (c.N <= kStepsNarrow)
+        return launch_pdl(ctx->pdl && !ctx->prof, dim3((c.N + 63) / 64, ns), dim3(32), ctx->stream,
+                          k_steps_pairs<DIP, 32, 1, 16>, c, crec, chunk, partial);
+      return launch_pdl(ctx->pdl && !ctx->prof, dim3((c.N + 511) / 512, ns), dim3(128), ctx->stream,
+                        k_steps_pairs<DIP, 128, 2, 4>, c, crec, chunk, partial);
     }));
     GBI_CHECK(launch_pdl(ctx->pdl && !ctx->prof, dim3(move), dim3(6 * kMoveSpheres), ctx->stream, k_steps_move<DIP>, c,
                          cpart, ns, R, p, rec));
