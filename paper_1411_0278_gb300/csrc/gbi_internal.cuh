@@ -128,11 +128,16 @@ inline bool balanced_form(int w) { return w == kFormTile || w == kFormChunk; }
 
 // Warps per target of the FP32 / double-float pair kernel: the requested value (2, 4,
 // 8 or 16; 1 selects the tiled form and 3 the chunk-balanced streaming form, which
-// serve one system only), else
-// enough warps to cover 152 SMs at small N and fewer (less reduction work per target)
-// once the N targets alone fill the GPU; capped by max_wpt.
+// serve one system only), else 4, or 2 in batches; capped by max_wpt.  With more warps per
+// target fewer blocks are resident, and a block's start (its positions' and first records'
+// latency) and final reduction overlap with fewer others; with fewer the last wave is coarser.  Whole
+// solves (mixed precision, us) with 2 / 4 / 8 / 16 warps: l <= 2 N = 500: 479 / 472 / 472 / 500, N = 2000: 1125 /
+// 1076 / 1157 / 1225, N = 12000: 20894 / 20430 / 21423; l <= 3 N = 1000: 968 / 960 / 993 / 1083, N = 9000: 34224 /
+// 33743 / 34168; l <= 4 N = 200: 682 / 602 / 647, N = 3000: 14832 / 14158 / 15073.  Batches, whose systems fill the
+// GPU together: 8 up to N = 300: 642 / 656 / 719 / 776, 48 up to 128: 701 / 746 / 905 / 1070, 48 up to 1024:
+// 2074 / 2154 / 2815 / 3422.
 inline int stream_wpt(int trunc, int precision, int N, int requested, bool batched = false) {
-  const int d = N >= 8192 ? 2 : (N >= 4096 ? 4 : (N >= 1024 ? 8 : 16));
+  const int d = batched ? 2 : 4;
   if (balanced_form(requested) && !batched && N > 1) return requested;
   const int w = (requested > 1 && !balanced_form(requested)) ? requested : d;
   const int cap = max_wpt(trunc, precision);

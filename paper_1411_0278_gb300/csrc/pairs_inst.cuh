@@ -92,7 +92,7 @@ cudaError_t launch_pairs_tt(int rows, int cols, const PairArgs& args, cudaStream
 #undef GBI_G
       return cudaErrorInvalidValue;
     }
-    const int wpt = stream_wpt(TRN, DF ? 2 : 1, N, args.wpt);
+    const int wpt = stream_wpt(TRN, DF ? 2 : 1, N, args.wpt, args.sys_of != nullptr && args.nsys > 1);
 #define GBI_S(RV, CV, WPT)                                                                         \
   if (rows == RV && cols == CV && wpt == WPT) {                                                    \
     constexpr int MINB = WARPS_SM / WPT > 0 ? WARPS_SM / WPT : 1;                                  \
