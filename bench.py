@@ -942,7 +942,7 @@ def run_ours(args):
                  "value": nw * N3 * (N3 - 1) / tw, "unit": UNIT, "image_terms_per_s": nw * N3 * N3 / tw,
                  "ms_per_evaluation": 1e3 * tw / nw,
                  "roofline": {"bound": "alu",
-                              "kernel": "wall images (records + k_wall_pairs<float>, nested dual numbers + reduce)",
+                              "kernel": "wall images (records + k_wall_pairs<float>, closed form + reduce)",
                               "achieved": achw, "peak": fp32_peak, "unit": "TFLOP/s", "frac": achw / fp32_peak,
                               "flops_per_image_term": sw["flops"] / max(1, sw["launches"]) / (N3 * N3),
                               "traffic": None, "avg_launch_ms": sw["ms"] / max(1, sw["launches"])},

@@ -380,7 +380,9 @@ __global__ void __launch_bounds__(kSmallThreads)
 template <bool DIP>
 gbi_status run_steps(gbi_ctx* ctx, const StepPar& c, int nsteps, double* R, double* p) {
   constexpr int W = StepRec<DIP>::W;
-  const double flops = trap_flops() * double(c.N) * double(c.N - 1);
+  // per pair: rho 9, r^2 5, rsqrt 1, powers 4, rho.F 5, S.rho 15, rho.S.rho 5, coefficients 11, V 18, Omega 30;
+  // the dipole 13 more
+  const double flops = (DIP ? 116.0 : 103.0) * double(c.N) * double(c.N - 1);
   const int ns = trap_splits(c.N, 1), chunk = (c.N + ns - 1) / ns;   // at most 2 splits up to kStepsSmall
   if (c.N <= kStepsSmall && !ctx->prof) {
     const int half = (c.N * ns + 31) / 32 * 32;   // threads of one kind of sum
