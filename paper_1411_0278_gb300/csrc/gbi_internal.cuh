@@ -128,16 +128,34 @@ inline bool balanced_form(int w) { return w == kFormTile || w == kFormChunk; }
 
 // Warps per target of the FP32 / double-float pair kernel: the requested value (2, 4,
 // 8 or 16; 1 selects the tiled form and 3 the chunk-balanced streaming form, which
-// serve one system only), else 4, or 2 in batches; capped by max_wpt.  With more warps per
+// serve one system only), else 4 or 8, or 2 in batches; capped by max_wpt.  With more warps per
 // target fewer blocks are resident, and a block's start (its positions' and first records'
 // latency) and final reduction overlap with fewer others; with fewer the last wave is coarser.  Whole
-// solves (mixed precision, us) with 2 / 4 / 8 / 16 warps: l <= 2 N = 500: 479 / 472 / 472 / 500, N = 2000: 1125 /
-// 1076 / 1157 / 1225, N = 12000: 20894 / 20430 / 21423; l <= 3 N = 1000: 968 / 960 / 993 / 1083, N = 9000: 34224 /
-// 33743 / 34168; l <= 4 N = 200: 682 / 602 / 647, N = 3000: 14832 / 14158 / 15073.  Batches, whose systems fill the
-// GPU together: 8 up to N = 300: 642 / 656 / 719 / 776, 48 up to 128: 701 / 746 / 905 / 1070, 48 up to 1024:
+// solves (mixed precision, us) with 2 / 4 / 8 / 16 warps: l <= 2 N = 2000: 1125 / 1076 / 1157 / 1225, N = 12000:
+// 20894 / 20430 / 21423; l <= 3 N = 1000: 968 / 960 / 993 / 1083, N = 9000: 34224 / 33743 / 34168; l <= 4
+// N = 200: 682 / 602 / 647, N = 3000: 14832 / 14158 / 15073.  Up to 1536 spheres, a few waves, the waves decide
+// between 4 and 8 (wave_cost): 4 / 8 warps l <= 2 N = 300: 452 / 428, N = 1000: 617 / 637; l <= 3 N = 700: 769 / 734;
+// l <= 4 N = 300: 686 / 750, 500: 1013 / 1077, 700: 1550 / 1512, 1000: 2355 / 2295.  Batches, whose systems fill
+// the GPU together: 8 up to N = 300: 642 / 656 / 719 / 776, 48 up to 128: 701 / 746 / 905 / 1070, 48 up to 1024:
 // 2074 / 2154 / 2815 / 3422.
+//
+// wave_cost: the waves of N targets over 152 SMs that hold `warps` warps each, times a block's rounds of
+// 32 w sources and its start and reduction (0.6 of a round); a last wave that leaves an SM with b of its B
+// blocks costs 0.6 + 0.4 b / B of a full one.
+inline long long wave_cost(int N, int w, int warps) {
+  const int B = warps / w > 0 ? warps / w : 1;
+  const long long slots = 152LL * B, full = N / slots, rest = N % slots;
+  const long long rounds = (N - 1 + 32 * w - 1) / (32 * w);
+  const long long b = (rest + 151) / 152;
+  return (20 * full + (rest > 0 ? 12 + 8 * b / B : 0)) * (5 * rounds + 3);
+}
+
 inline int stream_wpt(int trunc, int precision, int N, int requested, bool batched = false) {
-  const int d = batched ? 2 : 4;
+  int d = batched ? 2 : 4;
+  if (!batched && N <= 1536) {
+    const int warps = max_wpt(trunc, precision);   // resident per SM
+    if (wave_cost(N, 8, warps) < wave_cost(N, 4, warps)) d = 8;
+  }
   if (balanced_form(requested) && !batched && N > 1) return requested;
   const int w = (requested > 1 && !balanced_form(requested)) ? requested : d;
   const int cap = max_wpt(trunc, precision);
