@@ -49,8 +49,7 @@ struct gbi_ctx {
   bool allow_graphs = true;                      // run each GMRES cycle as one CUDA graph
   bool fixed = false;                            // buffers bound to static storage: never reallocate
   cudaGraphExec_t chunk_exec = nullptr;          // device-looped Arnoldi steps of one GMRES cycle
-  const void* chunk_key[8] = {};                 // buffers and sizes the graph was built for
-  long long chunk_ikey[8] = {};
+  std::vector<long long> chunk_key;              // sizes, radius and buffers the graph was built for
   int chunk_nodes = 0;                           // kernels per loop iteration
   // the whole mixed-precision solve as one graph: built when a call repeats the previous
   // call's key (buffers, sizes, parameters, tuning), replayed while the key stays

@@ -1432,6 +1432,13 @@ __global__ void bk_axpy_enabled(const double* __restrict__ d, int Ntot, const in
 // the triangular solves run on the device in FP64; the host launches the iterations
 // in chunks (replayed from a CUDA graph when the stream allows capture) and reads the
 // systems' small states once per chunk.
+// a double's bits, for the graphs' keys
+long long bits(double v) {
+  long long b;
+  std::memcpy(&b, &v, sizeof(b));
+  return b;
+}
+
 gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precision, const double* rhs, double* u,
                        bool u_is_zero, double tol, int restart, int max_iter, gbi_info* info, int& iters,
                        double& relres, GDev* hst, int* before, unsigned int* bar, double outer_rtol = 0.0);
@@ -1663,12 +1670,12 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
   // per-system states.  Built once per buffer set and replayed afterwards.
   const bool graphs = ctx->allow_graphs && ctx->stream != nullptr && !ctx->prof;
   if (graphs) {
-    const void* key[8] = {Vb, w, xsrc, ctx->gstate.p, B.sys, B.off, s.pos.hi, s.pos.p64};
-    const long long ikey[8] = {(long long)n, S, m, precision, s.trunc, Ntot, B.max_n, ctx->wpt_gen};
-    bool same = ctx->chunk_exec != nullptr;
-    for (int i = 0; i < 8 && same; ++i) same = ctx->chunk_key[i] == key[i];
-    for (int i = 0; i < 8 && same; ++i) same = ctx->chunk_ikey[i] == ikey[i];
-    if (!same) {
+    // what the captured launches hold: sizes, the radius (in the pair blocks and the
+    // preconditioner; the viscosity is in neither) and buffers
+    std::vector<long long> key = {(long long)n, S, m, precision, s.trunc, Ntot, B.max_n, ctx->wpt_gen, bits(s.a)};
+    const void* ptrs[] = {Vb, w, xsrc, ctx->gstate.p, B.sys, B.off, s.pos.hi, s.pos.p64};
+    for (const void* q : ptrs) key.push_back((long long)(uintptr_t)q);
+    if (ctx->chunk_exec == nullptr || key != ctx->chunk_key) {
       if (ctx->chunk_exec) cudaGraphExecDestroy(ctx->chunk_exec);
       ctx->chunk_exec = nullptr;
       cudaGraph_t graph = nullptr;
@@ -1700,8 +1707,7 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
       cudaGraphDestroy(graph);
       if (st != GBI_OK) return st;
       GBI_CHECK(e);
-      for (int i = 0; i < 8; ++i) ctx->chunk_key[i] = key[i];
-      for (int i = 0; i < 8; ++i) ctx->chunk_ikey[i] = ikey[i];
+      ctx->chunk_key = key;
     }
   }
   bool first = true;
@@ -2122,11 +2128,6 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
   const bool warm = warm_start != 0;
   if (prm->precision >= 1 && (!warm || hooks == nullptr) && ctx->allow_graphs && ctx->stream != nullptr &&
       !ctx->prof) {
-    auto bits = [](double v) {
-      long long b;
-      std::memcpy(&b, &v, sizeof(b));
-      return b;
-    };
     // the graph reads and writes only the context's own buffers (the caller's arrays are
     // packed before it and unpacked after it), so the key holds none of the caller's
     // every buffer the graph touches at its final size first (a repeated call then

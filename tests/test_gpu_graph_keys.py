@@ -1,0 +1,49 @@
+"""A context replays captured graphs of its solves; a call that differs in anything the captured
+launches hold must not get the old graph.  Every solve on the shared context is compared with the same
+solve on a context of its own.
+
+Tolerance: both solves end below a relative residual of 1e-10 with the same kernels: 1e-9 of the
+largest component (the preconditioned operator's condition number is below ~10)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _solve(gbi, ctx, R, p, a, trunc, precision, repeats=1):
+    i = ctx.trap_inputs(R.shape[0], trunc, 0.01, 0.1, 0.05, 0.02, R, p)
+    prm = gbi.params(a=a, eta=0.05, trunc=trunc, precision=precision, rtol=1e-10)
+    for _ in range(repeats):
+        out = ctx.solve(prm, R, i["Va"], i["Oa"], i["VH"], i["Fe"], i["Te"])
+    ctx.synchronize()
+    return out[:3]
+
+
+def _inputs(N, seed):
+    import torch
+    import workloads
+    s = workloads.small_cloud(N, seed, phi=0.05, dmin=2.3)
+    return [torch.tensor(np.ascontiguousarray(s[k]), dtype=torch.float64, device="cuda") for k in ("R", "p")]
+
+
+def _same(got, ref):
+    for x, y in zip(got, ref):
+        assert float((x - y).abs().max()) <= 1e-9 * max(float(y.abs().max()), 1e-6)
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("N", [60, 400])   # one-cluster step, separate kernels
+def test_another_radius(N, precision):
+    """The same suspension with spheres of another radius (no two overlap)."""
+    import torch
+    import paper_1411_0278_gb300 as gbi
+    R, p = _inputs(N, 3)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = gbi.Context(0, stream=stream)
+    for a in (1.0, 0.5, 1.1, 1.0):
+        got = _solve(gbi, ctx, R, p, a, 2, precision)
+        own = gbi.Context(0, stream=stream)
+        _same(got, _solve(gbi, own, R, p, a, 2, precision))
+        own.close()
+    ctx.close()
