@@ -24,6 +24,19 @@ struct df {
   __host__ __device__ explicit operator float() const { return hi; }
 };
 
+// A product whose rounding error is formed separately (fmaf(a, b, -p)): it must stay rounded.  Left
+// to itself the compiler may fuse it into a later sum -- s = p + e and e - (s - p) in df_fast_two_sum,
+// p - (s - v) in df_two_sum -- which then holds the product's error a second time, so that the value
+// is off by an FP32 rounding.  Whether it does depends on the code around it: the kernels as built were
+// not hit, the same block in another kernel was (l <= 3 H/L off by 1e-8 of its norm).
+__host__ __device__ __forceinline__ float df_rmul(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+
 __host__ __device__ __forceinline__ df df_two_sum(float a, float b) {
   const float s = a + b;
   const float v = s - a;
@@ -37,7 +50,7 @@ __host__ __device__ __forceinline__ df df_fast_two_sum(float a, float b) {
 }
 
 __host__ __device__ __forceinline__ df df_two_prod(float a, float b) {
-  const float p = a * b;
+  const float p = df_rmul(a, b);
   return df(p, fmaf(a, b, -p));
 }
 
@@ -54,7 +67,7 @@ __host__ __device__ __forceinline__ df operator-(df a) { return df(-a.hi, -a.lo)
 __host__ __device__ __forceinline__ df operator-(df a, df b) { return a + (-b); }
 
 __host__ __device__ __forceinline__ df operator*(df a, df b) {
-  const float p = a.hi * b.hi;
+  const float p = df_rmul(a.hi, b.hi);
   float e = fmaf(a.hi, b.hi, -p);
   e = fmaf(a.hi, b.lo, e);
   e = fmaf(a.lo, b.hi, e);
@@ -64,15 +77,6 @@ __host__ __device__ __forceinline__ df operator*(df a, df b) {
 __host__ __device__ __forceinline__ df& operator+=(df& a, df b) {
   a = a + b;
   return a;
-}
-
-// a product that the compiler must not fuse into a later sum
-__host__ __device__ __forceinline__ float df_rmul(float a, float b) {
-#ifdef __CUDA_ARCH__
-  return __fmul_rn(a, b);
-#else
-  return a * b;
-#endif
 }
 
 // a * b + c in 10 FP32 operations.  With p = fl(a.hi b.hi), s = fl(p + c.hi) and Knuth's split

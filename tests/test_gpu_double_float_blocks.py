@@ -1,0 +1,105 @@
+"""Double-float pair blocks against FP64 where the compiler sees them in another kernel than the
+library's: a program of its own, built here, whose kernels evaluate one block per thread.
+
+Bound: the error's measured rms over 2 to 3000 radii is at most 1.3e-13 of the block's norm and its largest
+value below 1e-11; an FP32 rounding that slips in is 1e-8.  1e-10 separates the two."""
+import os
+import subprocess
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1411_0278_gb300", "csrc")
+
+PROGRAM = r"""
+#include <cmath>
+#include <cstdio>
+#include <random>
+#include <vector>
+#include "df.cuh"
+#include "gbi_generated.cuh"
+#include "gbi_internal.cuh"
+#include "pair_kernel.cuh"
+using namespace gbi;
+
+// |double-float - FP64| of block x and the FP64 |block x|, for pair i
+template <int TR, int ROWS, int COLS>
+__global__ void k_block(int n, const double* rho, const double* x64, double* err, double* norm) {
+  using S = PassShape<TR, ROWS, COLS>;
+  constexpr int D = Tab<TR>::D;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  df xl[D], d[3], acc[S::NR];
+  double xd[D], dd[3], ad[S::NR];
+  for (int q = 0; q < S::NC; ++q) {
+    const float h = float(x64[64 * i + q]), l = float(x64[64 * i + q] - double(h));
+    xl[S::C0 + q] = df(h, l);
+    xd[S::C0 + q] = double(h) + double(l);
+  }
+  for (int k = 0; k < 3; ++k) {
+    const float h = float(rho[3 * i + k]), l = float(rho[3 * i + k] - double(h));
+    d[k] = df(h, l);
+    dd[k] = double(h) + double(l);
+  }
+  for (int p = 0; p < S::NR; ++p) {
+    acc[p] = df(0.f, 0.f);
+    ad[p] = 0.0;
+  }
+  pair_body<TR, ROWS, COLS, df>(d[0], d[1], d[2], df(1.f, 0.f), xl, acc);
+  pair_body<TR, ROWS, COLS, double>(dd[0], dd[1], dd[2], 1.0, xd, ad);
+  double e = 0.0, b = 0.0;
+  for (int p = 0; p < S::NR; ++p) {
+    const double v = df_to_double(acc[p]) - ad[p];
+    e += v * v;
+    b += ad[p] * ad[p];
+  }
+  err[i] = sqrt(e);
+  norm[i] = sqrt(b);
+}
+
+template <int TR, int ROWS, int COLS> int run(const char* name) {
+  const int n = 20000;
+  std::mt19937_64 g(7);
+  std::uniform_real_distribution<double> u(0.0, 1.0);
+  std::normal_distribution<double> z;
+  std::vector<double> rho(3 * n), x(64 * n), err(n), norm(n);
+  for (int i = 0; i < n; ++i) {
+    const double r = 2.0 * std::pow(1500.0, u(g)), v[3] = {z(g), z(g), (i % 2 ? 0.01 : 1.0) * z(g)};
+    const double s = r / std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+    for (int k = 0; k < 3; ++k) rho[3 * i + k] = s * v[k];
+    for (int q = 0; q < 64; ++q) x[64 * i + q] = z(g);
+  }
+  double *dr, *dx, *de, *dn;
+  cudaMalloc(&dr, 8 * 3 * n);
+  cudaMalloc(&dx, 8 * 64 * n);
+  cudaMalloc(&de, 8 * n);
+  cudaMalloc(&dn, 8 * n);
+  cudaMemcpy(dr, rho.data(), 8 * 3 * n, cudaMemcpyHostToDevice);
+  cudaMemcpy(dx, x.data(), 8 * 64 * n, cudaMemcpyHostToDevice);
+  k_block<TR, ROWS, COLS><<<(n + 127) / 128, 128>>>(n, dr, dx, de, dn);
+  if (cudaMemcpy(err.data(), de, 8 * n, cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
+  if (cudaMemcpy(norm.data(), dn, 8 * n, cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
+  double worst = 0.0;
+  for (int i = 0; i < n; ++i) worst = std::fmax(worst, err[i] / norm[i]);
+  std::printf("%s %.3e\n", name, worst);
+  return 0;
+}
+
+int main() {
+  return run<3, SET_H, SET_L>("l3_HL") || run<4, SET_H, SET_L>("l4_HL") || run<2, SET_H, SET_H>("l2_HH");
+}
+"""
+
+
+def test_blocks_in_another_kernel(tmp_path):
+    from paper_1411_0278_gb300 import build
+    src, exe = tmp_path / "blocks.cu", tmp_path / "blocks"
+    src.write_text(PROGRAM)
+    subprocess.run([build.nvcc(), "-std=c++17", "-O3", "-diag-suppress", "177"] + build.ARCH +
+                   ["-I", CSRC, str(src), "-o", str(exe)], check=True, capture_output=True)
+    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True, timeout=120).stdout
+    worst = {k: float(v) for k, v in (ln.split() for ln in out.splitlines())}
+    assert set(worst) == {"l3_HL", "l4_HL", "l2_HH"}
+    for name, w in worst.items():
+        assert w < 1e-10, (name, w)
