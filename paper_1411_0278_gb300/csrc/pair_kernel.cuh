@@ -92,7 +92,7 @@ __host__ __device__ __forceinline__ void dapplyT(const DMats<T>& dm, const T* in
 template <int J, typename T>
 __host__ __device__ __forceinline__ T eps_pow(const T* ep, T v) {
   if constexpr (J == 0) return v;
-  else return gbi_mul(ep[J], v);
+  else return ep[J] * v;
 }
 
 // Rotate the column modes [M, MEND) of x (absolute component index) into the pair
@@ -135,7 +135,7 @@ __host__ __device__ __forceinline__ void from_pair_frame(const T* yy, T* acc, co
     acc[o - R0 + k] = gbi_fmac(ep[l + 1], t[k], acc[o - R0 + k]);
 #pragma unroll
     for (int mm = 1; mm <= k; ++mm) {
-      const T c = gbi_mul(ep[l + 1], cm[mm]), s = gbi_mul(ep[l + 1], sm[mm]);
+      const T c = ep[l + 1] * cm[mm], s = ep[l + 1] * sm[mm];
       const T tp = t[k + mm], tn = t[k - mm];
       acc[o - R0 + k + mm] = gbi_fmac(c, tp, gbi_fmac(-s, tn, acc[o - R0 + k + mm]));
       acc[o - R0 + k - mm] = gbi_fmac(s, tp, gbi_fmac(c, tn, acc[o - R0 + k - mm]));

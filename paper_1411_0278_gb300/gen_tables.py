@@ -427,9 +427,10 @@ def factor(a):
     return a
 
 
-def fma_chain(terms):
+def fma_chain(terms, lean=False):
     """C++ expression for the sum of products [(a, b), ...] as a chain of gbi_fmac calls:
-    the first product is a plain multiply, every later one is fused into the sum."""
+    the first product is a plain multiply, every later one is fused into the sum.  lean: the first
+    product, if others follow, is a gbi_mul (left unnormalised in double-float)."""
     if not terms:
         return "T(0)"
     a0, b0 = terms[0]
@@ -437,6 +438,8 @@ def fma_chain(terms):
         expr = a0
     elif a0 in ("T(1.0)", "T(-1.0)"):
         expr = b0 if a0 == "T(1.0)" else "(-%s)" % b0
+    elif len(terms) == 1 or not lean:
+        expr = "%s * %s" % (a0, b0)
     else:
         expr = "gbi_mul(%s, %s)" % (factor(a0), b0)
     for a, b in terms[1:]:
@@ -486,7 +489,7 @@ def emit(path):
                     terms.append(("T(%s)" % fmt(v), mono))
             # put a constant term (no monomial) first, so that the chain starts from it
             terms.sort(key=lambda t: t[1] is not None)
-            w("  dm[%d] = %s;   // (mu=%d, nu=%d)" % (e, fma_chain(terms), mu, nu))
+            w("  dm[%d] = %s;   // (mu=%d, nu=%d)" % (e, fma_chain(terms, True), mu, nu))
         w("}")
         for transpose in (False, True):
             nm = "gbi_dapply%s%d" % ("T" if transpose else "", k)
@@ -500,7 +503,7 @@ def emit(path):
             for o in range(-k, k + 1):
                 terms = rows.get(o, [])
                 w("  out[%d] = %s;" % (o + k, fma_chain([("T(1.0)" if entries[e][1] == {(0, 0): 1} else "dm[%d]" % e,
-                                                             "in[%d]" % (i + k)) for e, i in terms])))
+                                                             "in[%d]" % (i + k)) for e, i in terms], True)))
             w("}")
     w("")
     # packing helpers for the trap inputs: U_mu . v^2 (mu = -2..2) and the Cartesian

@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1411_0278_gb300", "csrc")
 
 PROGRAM = r"""
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <random>
@@ -80,26 +81,45 @@ template <int TR, int ROWS, int COLS> int run(const char* name) {
   k_block<TR, ROWS, COLS><<<(n + 127) / 128, 128>>>(n, dr, dx, de, dn);
   if (cudaMemcpy(err.data(), de, 8 * n, cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
   if (cudaMemcpy(norm.data(), dn, 8 * n, cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
-  double worst = 0.0;
-  for (int i = 0; i < n; ++i) worst = std::fmax(worst, err[i] / norm[i]);
-  std::printf("%s %.3e\n", name, worst);
+  for (int i = 0; i < n; ++i) err[i] /= norm[i];
+  std::sort(err.begin(), err.end());
+  std::printf("%s %.3e %.3e\n", name, err[n / 2], err[n - 1]);
   return 0;
 }
 
 int main() {
-  return run<3, SET_H, SET_L>("l3_HL") || run<4, SET_H, SET_L>("l4_HL") || run<2, SET_H, SET_H>("l2_HH");
+  return run<3, SET_H, SET_L>("l3_HL") || run<4, SET_H, SET_L>("l4_HL") || run<2, SET_H, SET_H>("l2_HH") ||
+         run<3, SET_H, SET_H>("l3_HH");
 }
 """
 
 
-def test_blocks_in_another_kernel(tmp_path):
+# medians of the same program with every product normalised and 12 operations per fused product
+MEDIANS = {"l3_HL": 1.537e-14, "l4_HL": 1.593e-14, "l2_HH": 1.760e-14, "l3_HH": 1.979e-14}
+
+
+@pytest.fixture(scope="module")
+def blocks(tmp_path_factory):
+    """{block: (median, largest error)}"""
     from paper_1411_0278_gb300 import build
-    src, exe = tmp_path / "blocks.cu", tmp_path / "blocks"
+    d = tmp_path_factory.mktemp("blocks")
+    src, exe = d / "blocks.cu", d / "blocks"
     src.write_text(PROGRAM)
     subprocess.run([build.nvcc(), "-std=c++17", "-O3", "-diag-suppress", "177"] + build.ARCH +
                    ["-I", CSRC, str(src), "-o", str(exe)], check=True, capture_output=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True, timeout=120).stdout
-    worst = {k: float(v) for k, v in (ln.split() for ln in out.splitlines())}
-    assert set(worst) == {"l3_HL", "l4_HL", "l2_HH"}
-    for name, w in worst.items():
-        assert w < 1e-10, (name, w)
+    got = {k: (float(m), float(w)) for k, m, w in (ln.split() for ln in out.splitlines())}
+    assert set(got) == set(MEDIANS)
+    return got
+
+
+@pytest.mark.parametrize("name", sorted(MEDIANS))
+def test_blocks_in_another_kernel(blocks, name):
+    assert blocks[name][1] < 1e-10
+
+
+@pytest.mark.parametrize("name", sorted(MEDIANS))
+def test_cheaper_products_cost_no_accuracy(blocks, name):
+    """The typical error is no larger than with every product normalised (3%: the median of
+    20 000 pairs is known to about 1%)."""
+    assert blocks[name][0] <= 1.03 * MEDIANS[name]
