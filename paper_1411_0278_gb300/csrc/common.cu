@@ -589,12 +589,23 @@ gbi_status make_batch(gbi_ctx* ctx, int nsys, const int* offsets_host, Batch& B)
 // all the sources of a target at once, where the other forms give it two warps or more.  The
 // streaming form stays for larger systems (its lanes fill) and where a warps-per-target choice
 // is forced.
+//   Few rows (L): a lane's reduction and stores are short and the form wins wherever it fits; superposition in
+// double-float with two warps per target -> grouped, us: l <= 2 100 systems of 20: 64 -> 58, 400 of 33: 119 -> 105; l <= 4
+// 400 of 16: 133 -> 93, 400 of 33: 211 -> 168 (64 pairs of spheres: 61 -> 60).
+//   Rows H (the solves): every lane holds all the rows, so the reduction over many lanes costs more than
+// two warps' and a lane's serial stores more than the pairs it saves unless there are targets enough to hide
+// them.  Whole solves, streaming -> grouped, us: 1600 targets: l <= 2 200 systems of 8 476 -> 454, l <= 3 400 of 4
+// 625 -> 566, l <= 4 400 of 4 843 -> 688; 800: l <= 2 460 -> 459, l <= 3 400 of 2 558 -> 625, l <= 4 400 of 2 732 -> 795; 128:
+// l <= 4 599 -> 752.  16 lanes (16 spheres): 400 systems l <= 2 663 -> 610, l <= 3 984 -> 1115, l <= 4 1803 -> 1663; 32 lanes (20
+// spheres): l <= 2 705 -> 754, l <= 3 1111 -> 1686, l <= 4 2108 -> 2910.
 constexpr int kGroupMaxSystem = 33;
+constexpr int kGroupMinTargets = 1600;
 
-int group_lanes(const Batch& B) {
+int group_lanes(const Batch& B, int trunc, int rows) {
   if (B.S <= 1 || B.max_n > kGroupMaxSystem) return 0;
   int g = 1;
   while (g < B.max_n - 1) g <<= 1;
+  if (rows != SET_L && (B.Ntot < kGroupMinTargets || g > (trunc == 3 ? 8 : 16))) return 0;
   return g;
 }
 

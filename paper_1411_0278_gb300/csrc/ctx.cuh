@@ -243,8 +243,9 @@ struct Batch {
 bool valid_params(const gbi_params* p);
 // ordered pairs of a batch, sum over its systems of n (n - 1)
 long long batch_pairs(const Batch& B);
-// lanes per target of the group form for a batch, 0 where the other forms serve it
-int group_lanes(const Batch& B);
+// lanes per target of the group form for a batch's passes with these rows, 0 where the other
+// forms serve them
+int group_lanes(const Batch& B, int trunc, int rows);
 bool valid_offsets(int nsys, const int* off);
 gbi_status make_batch(gbi_ctx* ctx, int nsys, const int* offsets_host, Batch& B);
 gbi_status single_batch(gbi_ctx* ctx, int N, Batch& B);

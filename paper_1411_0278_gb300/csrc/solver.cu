@@ -1459,13 +1459,15 @@ constexpr long long kSysBlockElems = 4096;
 // ... and up to which a warp runs a system's whole step, norms included (bk_step_warp,
 // bk_norm_warp): eight elements per lane.  Used for batches of at least 64 systems, whose pair
 // passes then run in the group form (no warps-per-target choice forced).
-bool warp_systems(const gbi_ctx* ctx, const Batch& B, int h) {
-  return B.S >= 64 && (long long)B.max_n * h <= kWarpElems && ctx->force_wpt == 0 && group_lanes(B) > 0;
+bool warp_systems(const gbi_ctx* ctx, const Batch& B, int trunc) {
+  return B.S >= 64 && (long long)B.max_n * gbi_h(trunc) <= kWarpElems && ctx->force_wpt == 0 &&
+         group_lanes(B, trunc, SET_H) > 0;
 }
 
 // |x_s|^2 and what follows it (bk_norm_then), a warp per system where the systems are tiny
-void launch_norm(gbi_ctx* ctx, const Batch& B, int h, const GPtr& gp, const double* x, int mode, const NormCtl& nc) {
-  if (warp_systems(ctx, B, h))
+void launch_norm(gbi_ctx* ctx, const Batch& B, int trunc, const GPtr& gp, const double* x, int mode, const NormCtl& nc) {
+  const int h = gbi_h(trunc);
+  if (warp_systems(ctx, B, trunc))
     bk_norm_warp<<<(B.S + 3) / 4, 128, 0, ctx->stream>>>(x, B.Ntot, h, B.off, gp, mode, nc);
   else
     bk_norm_then<<<dim3(B.S, gp.CH), 256, 0, ctx->stream>>>(x, B.Ntot, h, B.off, gp, mode, nc);
@@ -1494,7 +1496,7 @@ constexpr int kArnoldiUnroll = 4;
 void launch_scale0(gbi_ctx* ctx, const Setup& s, const Batch& B, const GPtr& gp, double* Vb, const SrcOut& so,
                    int precision) {
   const size_t n = (size_t)B.Ntot * s.h;
-  if (!two_pass_gs(precision) && warp_systems(ctx, B, s.h))
+  if (!two_pass_gs(precision) && warp_systems(ctx, B, s.trunc))
     bk_scale0_warp<<<grid1(n), 256, 0, ctx->stream>>>(Vb, n, B.Ntot, s.h, B.sys, gp.st, so);
   else
     bk_scale0<<<dim3((B.Ntot + 255) / 256, s.h), 256, 0, ctx->stream>>>(Vb, B.Ntot, B.sys, gp.st, so);
@@ -1503,7 +1505,7 @@ void launch_scale0(gbi_ctx* ctx, const Setup& s, const Batch& B, const GPtr& gp,
 void launch_update(gbi_ctx* ctx, const Setup& s, const Batch& B, const GPtr& gp, const double* Vb, double* u,
                    int precision) {
   const size_t n = (size_t)B.Ntot * s.h;
-  if (!two_pass_gs(precision) && warp_systems(ctx, B, s.h))
+  if (!two_pass_gs(precision) && warp_systems(ctx, B, s.trunc))
     bk_update_warp<<<grid1(n), 256, 0, ctx->stream>>>(Vb, n, B.Ntot, s.h, B.sys, gp, s.minv, u);
   else
     bk_update<<<dim3((B.Ntot + 255) / 256, s.h), 256, 0, ctx->stream>>>(Vb, n, B.Ntot, B.sys, gp, s.minv, u);
@@ -1530,13 +1532,13 @@ gbi_status launch_chunk(gbi_ctx* ctx, const Setup& s, const Batch& B, int precis
   pa.nsys = B.S;
   pa.npairs = batch_pairs(B);
   pa.sys_off = B.off;
-  pa.group = group_lanes(B);
+  pa.group = group_lanes(B, s.trunc, SET_H);
   pa.sys_flag = &gp.st[0].active;
   pa.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
   const SrcOut so = src_out(s, precision, xsrc);
   const dim3 gd(S, m + 1, gp.CH);
   const int two = two_pass_gs(precision);
-  pa.y_sphere = !two && warp_systems(ctx, B, h) ? 1 : 0;
+  pa.y_sphere = !two && warp_systems(ctx, B, s.trunc) ? 1 : 0;
   // programmatic dependent launch inside the one-reduction step, between kernels of the
   // same sequence (the first pair pass of a chunk follows other work)
   const bool pdl = ctx->pdl && !two;
@@ -1580,7 +1582,7 @@ gbi_status launch_chunk(gbi_ctx* ctx, const Setup& s, const Batch& B, int precis
       bk_finalize<<<S, 128, 0, ctx->stream>>>(gp, 1);
       bk_scale<<<g2, 256, 0, ctx->stream>>>(Vb, n, w, Ntot, B.sys, gp.st, so, lcs);
       ctx->launches += 7;
-    } else if (warp_systems(ctx, B, h)) {
+    } else if (warp_systems(ctx, B, s.trunc)) {
       // many tiny systems: a warp runs the rest of a system's step
       GBI_CHECK(launch_pdl_smem(pdl, dim3((S + kStepWarps - 1) / kStepWarps), dim3(32 * kStepWarps),
                                 sizeof(double) * kStepWarps * (3 * m + 2), ctx->stream, bk_step_warp, Vb, n, w, Ntot,
@@ -1721,7 +1723,7 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
       pr.nsys = B.S;
       pr.npairs = batch_pairs(B);
       pr.sys_off = B.off;
-      pr.group = group_lanes(B);
+      pr.group = group_lanes(B, s.trunc, SET_H);
       pr.sys_flag = &gp.st[0].enabled;
       pr.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
       GBI_CHECK(run_pairs(ctx, s.trunc, SET_H, SET_H, precision, pr));
@@ -1735,7 +1737,7 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
       NormCtl nc{};
       nc.follow = kFollowCycle;
       nc.first = first ? 1 : 0;
-      launch_norm(ctx, B, h, gp, Vb, 1, nc);
+      launch_norm(ctx, B, s.trunc, gp, Vb, 1, nc);
     }
     launch_scale0(ctx, s, B, gp, Vb, src_out(s, precision, xsrc), precision);
     GBI_CHECK(cudaGetLastError());
@@ -1985,7 +1987,7 @@ gbi_status emit_gmres(GraphBuild& gb, const Setup& s, const Batch& B, const GPtr
     pr.nsys = B.S;
     pr.npairs = batch_pairs(B);
     pr.sys_off = B.off;
-    pr.group = group_lanes(B);
+    pr.group = group_lanes(B, s.trunc, SET_H);
     pr.sys_flag = &gp.st[0].enabled;
     pr.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
     pr.active = &d->notfirst;   // u is zero in the first cycle
@@ -1996,7 +1998,7 @@ gbi_status emit_gmres(GraphBuild& gb, const Setup& s, const Batch& B, const GPtr
       nc.follow = kFollowCycle;
       nc.d = d;
       nc.ha = ha;
-      launch_norm(ctx, B, h, gp, Vb, 1, nc);
+      launch_norm(ctx, B, s.trunc, gp, Vb, 1, nc);
     }
     launch_scale0(ctx, s, B, gp, Vb, src_out(s, 1, xsrc), 1);
     GBI_TRY(gb.body(gb.node(ha, cudaGraphCondTypeWhile), kBodyStep, [&]() -> gbi_status {
@@ -2055,12 +2057,12 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
   const double c2a = s.scale.v[3];
   Scales hscale;
   for (int i = 0; i < kMaxD; ++i) hscale.v[i] = (i < h) ? s.scale.v[6 + i] : 1.0;
-  auto batched = [&](PairArgs p, const int* flag) {
+  auto batched = [&](PairArgs p, const int* flag, int rows = SET_H) {
     p.sys_of = B.sys;
     p.nsys = B.S;
     p.npairs = batch_pairs(B);
     p.sys_off = B.off;
-    p.group = group_lanes(B);
+    p.group = group_lanes(B, s.trunc, rows);
     p.sys_flag = flag;
     p.sys_flag_stride = int(sizeof(GDev) / sizeof(int));
     return p;
@@ -2101,7 +2103,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
   auto output_pass = [&]() -> gbi_status {
     PairArgs p = batched(pair_args(s, P<double>(ctx->xQ), P<double>(ctx->xVL), -1.0 / (8.0 * kPi * s.eta), 0.0, 1,
                                    s.ones, 0),
-                         nullptr);
+                         nullptr, SET_L);
     GBI_CHECK(run_pairs(ctx, s.trunc, SET_L, SET_ALL, io, p));
     return GBI_OK;
   };
@@ -2191,7 +2193,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
                 NormCtl nc{};
                 nc.follow = kFollowRefine0;
                 nc.rtol = rtol;
-                launch_norm(ctx, B, h, gp, b, 2, nc);
+                launch_norm(ctx, B, s.trunc, gp, b, 2, nc);
               }
               gk_guard<<<1, 256, 0, ctx->stream>>>(gp, P<unsigned int>(ctx->minr2), bad_in, s.a,
                                                    pairs_all > 0 ? prm->min_sep : 0.0, d);
@@ -2213,7 +2215,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
                 NormCtl nc{};
                 nc.follow = kFollowWarm;
                 nc.rtol = rtol;
-                launch_norm(ctx, B, h, gp, r, 1, nc);
+                launch_norm(ctx, B, s.trunc, gp, r, 1, nc);
                 GBI_CHECK(cudaMemsetAsync(dl, 0, sizeof(double) * nh, ctx->stream));
                 GBI_TRY(emit_gmres(gb, s, B, gp, restart, r, dl, inner, max_iter, rtol, d));
                 bk_axpy_enabled<<<g2, 256, 0, ctx->stream>>>(dl, N, B.sys, gp.st, xQH);
@@ -2250,7 +2252,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
                   nc.max_refine = max_refine;
                   nc.max_iter = max_iter;
                   nc.incr = incr ? 1 : 0;
-                  launch_norm(ctx, B, h, gp, r, 1, nc);
+                  launch_norm(ctx, B, s.trunc, gp, r, 1, nc);
                 }
                 GBI_CHECK(cudaGetLastError());
                 return gb.body(gb.node(hif, cudaGraphCondTypeIf), kBodyIf, [&]() -> gbi_status {
@@ -2382,7 +2384,7 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
     NormCtl nc{};
     nc.follow = follow;
     nc.rtol = rtol;
-    launch_norm(ctx, B, h, gp, x, mode, nc);
+    launch_norm(ctx, B, s.trunc, gp, x, mode, nc);
   };
   norm_refine(b, 2, kFollowRefine0);
   auto read_state = [&]() -> gbi_status {
