@@ -425,15 +425,20 @@ gbi_status gbi_mlp_labels_qh(gbi_ctx* ctx, int N, int h, double s0, const double
                              double* sigma, double* labels);
 
 /* Tuning of the pair kernel (engineering; the paper has no counterpart).  The FP32
- * and double-float pair passes run in one of two forms.  Streaming: one block per
+ * and double-float pair passes run in one of these forms.  Streaming: one block per
  * target sphere whose WPT warps split the sources; WPT in {2, 4, 8, 16} (8 at most for
  * trunc 4 and double-float) trades parallelism at small N against per-target
  * reduction work.  Tiled (code WPT = 1, one system only, not batches): lanes are 32
  * target spheres, source records are staged in shared memory by the TMA unit and read
  * by all lanes at once, and the (targets, source) work is split evenly over one block
  * per SM; the blocks' partial sums are added in a fixed order, so results do not
- * depend on timing.  Both forms sum the same pairs (in different fixed orders).
- * gbi_tune times every WPT for the six FP32 / double-float passes of the mixed-precision
+ * depend on timing.  Grouped (code WPT = 32, batches whose systems have at most 33
+ * spheres): a few lanes share a target, several targets a warp.  It is the untuned choice
+ * of such batches for rows L, and for rows H from 1600 spheres on where 16 lanes (8 for
+ * trunc 3) hold a target's sources.  All forms sum the same pairs (in different fixed
+ * orders).
+ * gbi_tune times every WPT (the grouped form too where the layout's passes would take it)
+ * for the six FP32 / double-float passes of the mixed-precision
  * solves -- rows H / columns H in FP32 and in double-float, H/L and L/all in
  * double-float, H/L and L/all in FP32 -- on synthetic
  * input of the given layout: nsys systems, system s holding spheres
@@ -447,7 +452,9 @@ gbi_status gbi_mlp_labels_qh(gbi_ctx* ctx, int N, int h, double s0, const double
  * buffers and synchronizes the stream (not capturable).
  * gbi_set_wpt forces one WPT for every later pass (0 = back to tuned/default).
  * gbi_pass_wpt returns the WPT a pass with these parameters would use (0 for the
- * FP64 tiled pass, -1 for invalid arguments).
+ * FP64 tiled pass, -1 for invalid arguments).  For batches it does not know the systems: 32
+ * stands for the grouped form where they suit it and the untuned streaming choice where not,
+ * and an untuned batch that suits the grouped form takes that instead of the value returned.
  * Split tail (streaming form, one system; off by default): when the N target blocks do not
  * fill whole waves of the resident block slots, the targets of the last, partly filled
  * wave have their sources split into 2..8 blocks each (the count that best fills the

@@ -347,7 +347,8 @@ class Context:
     def tune(self, trunc, offsets, reps=0):
         """gbi_tune: time each warps-per-target choice of the pair passes on synthetic
         input with the sphere layout ``offsets`` (nsys + 1 ints); returns the 6 choices
-        (H/H FP32, H/H double-float, H/L and L/all double-float, H/L and L/all FP32)."""
+        (H/H FP32, H/H double-float, H/L and L/all double-float, H/L and L/all FP32; 32: the
+        grouped form of batches of small systems)."""
         off = _c_ints(offsets)
         out = (ctypes.c_int * 6)()
         self._check(lib().gbi_tune(self._h, int(trunc), len(offsets) - 1, off, int(reps), out), "gbi_tune")

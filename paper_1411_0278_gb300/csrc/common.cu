@@ -294,7 +294,8 @@ cudaError_t run_pairs(gbi_ctx* ctx, int trunc, int rows, int cols, int precision
     args.wpt = ctx->force_wpt > 0 ? ctx->force_wpt
                                   : ctx->tuned_wpt(trunc, rows, cols, precision, args.N,
                                                    args.sys_of != nullptr && args.nsys > 1);
-  if (precision == 0 || ctx->force_wpt > 0) args.group = 0;
+  if (precision == 0 || !ctx->group_allowed(trunc, rows, cols, precision, args.N)) args.group = 0;
+  if (args.wpt == kFormGroup) args.wpt = 0;   // where the batch's systems do not suit it: the default
   tile_select(ctx, trunc, rows, precision, args);
   if (precision >= 1 && !balanced_form(args.wpt) && !(args.sys_of != nullptr && args.nsys > 1) &&
       ctx->split_tail)
@@ -588,7 +589,7 @@ gbi_status make_batch(gbi_ctx* ctx, int nsys, const int* offsets_host, Batch& B)
 // The group form serves batches whose every system has at most 33 spheres: a warp then holds
 // all the sources of a target at once, where the other forms give it two warps or more.  The
 // streaming form stays for larger systems (its lanes fill) and where a warps-per-target choice
-// is forced.
+// is forced or was tuned.
 //   Few rows (L): a lane's reduction and stores are short and the form wins wherever it fits; superposition in
 // double-float with two warps per target -> grouped, us: l <= 2 100 systems of 20: 64 -> 58, 400 of 33: 119 -> 105; l <= 4
 // 400 of 16: 133 -> 93, 400 of 33: 211 -> 168 (64 pairs of spheres: 61 -> 60).

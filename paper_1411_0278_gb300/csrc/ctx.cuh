@@ -103,6 +103,11 @@ struct gbi_ctx {
     const auto it = wpt_table.find(wpt_key(trunc, rows, cols, precision, N, batched));
     return it == wpt_table.end() ? 0 : it->second;
   }
+  // a batch's pass may take the grouped form: nothing forced, and nothing else tuned for it
+  bool group_allowed(int trunc, int rows, int cols, int precision, int N) const {
+    const int w = tuned_wpt(trunc, rows, cols, precision, N, true);
+    return force_wpt == 0 && (w == 0 || w == gbi::kFormGroup);
+  }
 };
 
 namespace gbi {

@@ -127,6 +127,10 @@ gbi_status tune_impl(gbi_ctx* ctx, int trunc, int nsys, const int* offsets, int 
   const int D = d_of(trunc);
   const int Ntot = offsets[nsys];
   const bool batched = nsys > 1;
+  Batch layout;
+  layout.S = nsys;
+  layout.Ntot = Ntot;
+  for (int q = 0; q < nsys; ++q) layout.max_n = std::max(layout.max_n, offsets[q + 1] - offsets[q]);
   TuneBufs tb;
   const int rf_max = rec_floats(D, true);
   GBI_CHECK(cudaMalloc(&tb.p[0], sizeof(float4) * Ntot));
@@ -179,17 +183,20 @@ gbi_status tune_impl(gbi_ctx* ctx, int trunc, int nsys, const int* offsets, int 
     pa.x32 = rec;
     int best = 0;
     float best_ms = 0.f;
-    // candidates: the tiled form (1, one system only) and 2, 4, ... warps per target of
-    // the streaming form
+    // candidates: the tiled form (1, one system only), 2, 4, ... warps per target of the
+    // streaming form, and the grouped form where such a batch's passes would take it
     std::vector<int> cand;
     if (!batched) {
       cand.push_back(kFormTile);
       cand.push_back(kFormChunk);
     }
     for (int w = 2; w <= max_wpt(trunc, ps.precision); w *= 2) cand.push_back(w);
+    const int lanes = group_lanes(layout, trunc, ps.rows);
+    if (lanes > 0) cand.push_back(kFormGroup);
     for (const int w : cand) {
       if (e != cudaSuccess) break;
-      pa.wpt = w;
+      pa.wpt = w == kFormGroup ? 0 : w;
+      pa.group = w == kFormGroup ? lanes : 0;
       pa.nsplit = 0;
       if (balanced_form(w) && !balanced_args(ctx, trunc, ps.rows, ps.precision, Ntot, pa)) continue;
       if (!balanced_form(w) && !batched && ctx->split_tail) split_reserve(ctx, trunc, ps.rows, ps.precision, pa);
@@ -676,7 +683,7 @@ int gbi_pass_wpt(gbi_ctx* ctx, int trunc, int rows, int cols, int precision, int
   if (precision == 0) return 0;
   if ((precision != 1 && precision != 2) || fp64_only(trunc)) return -1;
   const int req = ctx->force_wpt > 0 ? ctx->force_wpt : ctx->tuned_wpt(trunc, rows, cols, precision, N, batched != 0);
-  return stream_wpt(trunc, precision, N, req, batched != 0);
+  return req == kFormGroup ? req : stream_wpt(trunc, precision, N, req, batched != 0);
 }
 
 gbi_status gbi_set_profiling(gbi_ctx* ctx, int on) {

@@ -124,6 +124,7 @@ inline int max_wpt(int trunc, int precision) { return (trunc == 4 || precision =
 // Code of the tiled form of pair_tile.cuh (lanes are targets; single systems only).
 constexpr int kFormTile = 1;
 constexpr int kFormChunk = 3;   // chunk-balanced streaming form (pair_chunk.cuh), one system
+constexpr int kFormGroup = 32;  // grouped form (pair_group_kernel), batches of small systems
 inline bool balanced_form(int w) { return w == kFormTile || w == kFormChunk; }
 
 // Warps per target of the FP32 / double-float pair kernel: the requested value (2, 4,

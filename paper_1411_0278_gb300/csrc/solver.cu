@@ -1458,10 +1458,10 @@ SrcOut src_out(const Setup& s, int precision, void* xsrc) {
 constexpr long long kSysBlockElems = 4096;
 // ... and up to which a warp runs a system's whole step, norms included (bk_step_warp,
 // bk_norm_warp): eight elements per lane.  Used for batches of at least 64 systems, whose pair
-// passes then run in the group form (no warps-per-target choice forced).
+// passes then run in the group form (no warps-per-target choice forced or tuned).
 bool warp_systems(const gbi_ctx* ctx, const Batch& B, int trunc) {
-  return B.S >= 64 && (long long)B.max_n * gbi_h(trunc) <= kWarpElems && ctx->force_wpt == 0 &&
-         group_lanes(B, trunc, SET_H) > 0;
+  return B.S >= 64 && (long long)B.max_n * gbi_h(trunc) <= kWarpElems && group_lanes(B, trunc, SET_H) > 0 &&
+         ctx->group_allowed(trunc, SET_H, SET_H, 1, B.Ntot);
 }
 
 // |x_s|^2 and what follows it (bk_norm_then), a warp per system where the systems are tiny

@@ -91,3 +91,36 @@ def test_warm_start(trunc, sizes, precision):
             for x, y in zip(got[:3], ref):
                 close(x, y, 1e-8 if precision < 3 else 1e-5)
     ctx.close()
+
+
+def test_tuned_choice_is_kept():
+    """What gbi_tune chose for a batch's passes serves every later batch of that size class: the pass
+    gives the bits of the same choice forced (sums of 16 sources in another order differ)."""
+    gbi, ctx, R, offs, a = _case(2, [17] * 130)
+    prm = gbi.params(a=1.0, eta=0.7, trunc=2, precision=1)
+    chosen = ctx.tune(2, [130 * k for k in range(18)], reps=2)   # 17 systems of 130: streaming forms only
+    assert all(w in (2, 4, 8, 16) for w in chosen)
+    assert ctx.pass_wpt(2, 1, 0, 1, offs[-1], batched=True) == chosen[5]
+    got = ctx.batch_superpose(prm, offs, R, *a)
+    ctx.set_wpt(chosen[5])
+    for x, y in zip(got, ctx.batch_superpose(prm, offs, R, *a)):
+        assert bool((x == y).all())
+    ctx.close()
+
+
+@pytest.mark.parametrize("trunc,sizes", [(2, [17] * 130), (4, [3, 2] * 400), (4, [17, 20] * 10)])
+def test_tuning_a_batch_of_small_systems(trunc, sizes):
+    """The grouped form is a candidate, reported as 32 and kept; results stay."""
+    gbi, ctx, R, offs, a = _case(trunc, sizes)
+    prm = gbi.params(a=1.0, eta=0.7, trunc=trunc, precision=2, rtol=1e-10)
+    ref = ctx.batch_solve(prm, offs, R, *a)[:3]
+    chosen = ctx.tune(trunc, offs, reps=2)
+    assert all(w in (2, 4, 8, 16, 32) for w in chosen)
+    passes = [(2, 2, 1), (2, 2, 2), (2, 1, 2), (1, 0, 2), (2, 1, 1), (1, 0, 1)]
+    for (rows, cols, precision), w in zip(passes, chosen):
+        assert ctx.pass_wpt(trunc, rows, cols, precision, offs[-1], batched=True) == w
+    for _ in range(3):
+        got = ctx.batch_solve(prm, offs, R, *a)[:3]
+    for x, y in zip(got, ref):
+        close(x, y, 1e-8)
+    ctx.close()
