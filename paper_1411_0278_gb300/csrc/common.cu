@@ -74,6 +74,13 @@ gbi_status ensure(gbi_ctx* ctx, Buf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (b.bytes >= bytes) return GBI_OK;
   if (ctx->fixed) return GBI_ERR_NOMEM;   // static storage: never reallocated
+  // inside a capture nothing can be allocated or waited for, and trying ends the capture
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (ctx->stream != nullptr && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess &&
+      cap != cudaStreamCaptureStatusNone) {
+    ctx->err = "the workspace would have to grow inside a stream capture";
+    return GBI_ERR_CUDA;
+  }
   if (b.p) {
     GBI_CHECK(cudaStreamSynchronize(ctx->stream));
     GBI_CHECK(cudaFree(b.p));
@@ -285,21 +292,33 @@ bool split_reserve(gbi_ctx* ctx, int trunc, int rows, int precision, PairArgs& a
   return true;
 }
 
+// The form of a pass (forced, tuned or default) with its plan and scratch
+static void select_form(gbi_ctx* ctx, int trunc, int rows, int cols, int precision, PairArgs& args) {
+  const bool batched = args.sys_of != nullptr && args.nsys > 1;
+  if (args.wpt == 0)
+    args.wpt = ctx->force_wpt > 0 ? ctx->force_wpt
+                                  : ctx->tuned_wpt(trunc, rows, cols, precision, args.N, batched);
+  if (precision == 0 || !ctx->group_allowed(trunc, rows, cols, precision, args.N)) args.group = 0;
+  if (args.wpt == kFormGroup) args.wpt = 0;   // where the batch's systems do not suit it: the default
+  tile_select(ctx, trunc, rows, precision, args);
+  if (precision >= 1 && !balanced_form(args.wpt) && !batched && ctx->split_tail)
+    split_reserve(ctx, trunc, rows, precision, args);
+}
+
+void reserve_pass(gbi_ctx* ctx, int trunc, int rows, int cols, int precision, int N) {
+  if (precision == 0) return;
+  PairArgs args{};
+  args.N = N;
+  args.nsys = 1;
+  select_form(ctx, trunc, rows, cols, precision, args);
+}
+
 cudaError_t run_pairs(gbi_ctx* ctx, int trunc, int rows, int cols, int precision, const PairArgs& args_in) {
   const double pairs = args_in.npairs > 0 ? double(args_in.npairs) : double(args_in.N) * double(args_in.N - 1);
   const double flops = pair_flops(trunc, rows, cols) * pairs;
   PairArgs args = args_in;
   int extra = 0;
-  if (args.wpt == 0)
-    args.wpt = ctx->force_wpt > 0 ? ctx->force_wpt
-                                  : ctx->tuned_wpt(trunc, rows, cols, precision, args.N,
-                                                   args.sys_of != nullptr && args.nsys > 1);
-  if (precision == 0 || !ctx->group_allowed(trunc, rows, cols, precision, args.N)) args.group = 0;
-  if (args.wpt == kFormGroup) args.wpt = 0;   // where the batch's systems do not suit it: the default
-  tile_select(ctx, trunc, rows, precision, args);
-  if (precision >= 1 && !balanced_form(args.wpt) && !(args.sys_of != nullptr && args.nsys > 1) &&
-      ctx->split_tail)
-    split_reserve(ctx, trunc, rows, precision, args);
+  select_form(ctx, trunc, rows, cols, precision, args);
   if (precision == 2 || (precision == 1 && args.x32 == nullptr)) {
     // per-sphere source records (FP32, or the double-float hi/lo pair), once per pass,
     // so that the pair loop touches no FP64

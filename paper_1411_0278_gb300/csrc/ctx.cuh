@@ -132,7 +132,8 @@ gbi_status fail(gbi_ctx* c, cudaError_t e, const char* where);
 
 // at least `bytes` of host scratch in ctx->hs (never shrinks; refuses for static storage)
 gbi_status host_scratch(gbi_ctx* ctx, size_t bytes);
-// grow a workspace buffer to at least `bytes` (never shrinks; refuses for static storage)
+// grow a workspace buffer to at least `bytes` (never shrinks; refuses for static storage and
+// while the context's stream is being captured)
 gbi_status ensure(gbi_ctx* ctx, Buf& b, size_t bytes);
 template <typename T> T* P(Buf& b) { return reinterpret_cast<T*>(b.p); }
 
@@ -189,6 +190,8 @@ bool balanced_args(gbi_ctx* ctx, int trunc, int rows, int precision, int N, Pair
 // PairArgs) and its scratch in the context; false (and no split) if it does not pay or its
 // scratch cannot be had
 bool split_reserve(gbi_ctx* ctx, int trunc, int rows, int precision, PairArgs& a);
+// the scratch of a one-system pass's form ahead of a capture, in which nothing can be allocated
+void reserve_pass(gbi_ctx* ctx, int trunc, int rows, int cols, int precision, int N);
 cudaError_t run_trap(gbi_ctx* ctx, const TrapArgs& t, int precision);
 // nsteps Euler steps of one suspension in a trap by the l <= 2 superposition in FP32 (trap_steps.cu)
 gbi_status superposition_steps(gbi_ctx* ctx, const gbi_params* prm, int N, double dt, double k_trap, double vs,

@@ -2122,6 +2122,14 @@ gbi_status solve_core(gbi_ctx* ctx, const gbi_params* prm, const Batch& B, const
   const double rtol = prm->rtol > 0 ? prm->rtol : 1e-10;
   const double inner = prm->inner_rtol > 0 ? prm->inner_rtol : 1e-5;
   const int max_refine = prm->max_refine > 0 ? prm->max_refine : 8;
+  if (S == 1 && prm->precision >= 1) {
+    // the passes' scratch (balanced forms, split tails), ahead of the graphs' captures: a capture may
+    // come before the pass has run
+    reserve_pass(ctx, s.trunc, SET_H, SET_L, io, N);
+    reserve_pass(ctx, s.trunc, SET_H, SET_H, hp, N);
+    reserve_pass(ctx, s.trunc, SET_H, SET_H, 1, N);
+    reserve_pass(ctx, s.trunc, SET_L, SET_ALL, io, N);
+  }
 
   // ---- the mixed-precision solve as one graph (see GraphBuild): every device step of
   // the sequence below, the decisions taken by kernels instead of the host

@@ -47,3 +47,29 @@ def test_another_radius(N, precision):
         _same(got, _solve(gbi, own, R, p, a, 2, precision))
         own.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("N,trunc,precision,wpt", [(642, 3, 2, 0), (1000, 3, 2, 0), (1000, 3, 3, 0), (1024, 3, 1, 0),
+                                                   (300, 2, 1, 1), (300, 2, 1, 3), (300, 2, 3, 1)])
+def test_scratch_before_the_capture(N, trunc, precision, wpt):
+    """A fresh context captures the FP32 pass of its first solve before that pass has run; the split
+    tail's and the balanced forms' scratch has to be there (forced forms, and sizes at which the
+    FP32 pass needs more of it than the double-float one)."""
+    import torch
+    import paper_1411_0278_gb300 as gbi
+    R, p = _inputs(N, 5)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    plain = gbi.Context(0, stream=stream)
+    ref = _solve(gbi, plain, R, p, 1.0, trunc, precision)
+    plain.close()
+    ctx = gbi.Context(0, stream=stream)
+    ctx.set_split_tail(1)
+    ctx.set_wpt(wpt)
+    for _ in range(3):       # direct, capture, replay
+        got = _solve(gbi, ctx, R, p, 1.0, trunc, precision)
+        for x, y in zip(got, ref):
+            tol = 1e-9 if precision < 3 else 1e-5
+            assert float((x - y).abs().max()) <= tol * float(y.abs().max())
+    assert ctx.solve_graph_replays() >= 1
+    ctx.close()
