@@ -1675,7 +1675,8 @@ gbi_status gmres_batch(gbi_ctx* ctx, const Setup& s, const Batch& B, int precisi
     // what the captured launches hold: sizes, the radius (in the pair blocks and the
     // preconditioner; the viscosity is in neither) and buffers
     std::vector<long long> key = {(long long)n, S, m, precision, s.trunc, Ntot, B.max_n, ctx->wpt_gen, bits(s.a)};
-    const void* ptrs[] = {Vb, w, xsrc, ctx->gstate.p, B.sys, B.off, s.pos.hi, s.pos.p64};
+    const void* ptrs[] = {Vb, w, xsrc, ctx->gstate.p, B.sys, B.off, s.pos.hi, s.pos.lo, s.pos.p64, ctx->minr2.p,
+                          ctx->tile.p, ctx->tilecnt.p};
     for (const void* q : ptrs) key.push_back((long long)(uintptr_t)q);
     if (ctx->chunk_exec == nullptr || key != ctx->chunk_key) {
       if (ctx->chunk_exec) cudaGraphExecDestroy(ctx->chunk_exec);

@@ -73,3 +73,26 @@ def test_scratch_before_the_capture(N, trunc, precision, wpt):
             assert float((x - y).abs().max()) <= tol * float(y.abs().max())
     assert ctx.solve_graph_replays() >= 1
     ctx.close()
+
+
+def test_scratch_that_moves_between_solves():
+    """A larger pass grows (and moves) the split tail's scratch while every other buffer stays: the next
+    solve's steps must use the new one."""
+    import torch
+    import paper_1411_0278_gb300 as gbi
+    N, trunc = 1000, 3
+    R, p = _inputs(N, 6)
+    big, _ = _inputs(3040, 7)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        torch.cuda.synchronize()
+        ctx = gbi.Context(0, stream=stream)
+        ctx.set_split_tail(1)
+        x = torch.randn(25, 3040, dtype=torch.float64, device="cuda")
+        y = torch.zeros_like(x)
+        ctx.apply(3040, trunc, 1.0, 2, 2, 1, big, x, y)      # five full waves: buffers for 3040, no split
+        ref = _solve(gbi, ctx, R, p, 1.0, trunc, 2)
+        ctx.apply(2900, trunc, 1.0, 2, 2, 1, big, x, y)      # a tail of 468 targets in five parts
+        for _ in range(3):
+            _same(_solve(gbi, ctx, R, p, 1.0, trunc, 2), ref)
+        ctx.close()
