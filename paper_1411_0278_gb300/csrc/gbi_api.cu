@@ -659,6 +659,7 @@ gbi_status gbi_set_split_tail(gbi_ctx* ctx, int on) {
 gbi_status gbi_set_wait_limit(gbi_ctx* ctx, long long rounds) {
   if (!ctx || rounds < -1) return GBI_ERR_ARG;
   ctx->wait_limit = rounds == -1 ? kTileWaitLimit : rounds;
+  ++ctx->wpt_gen;   // captured graphs hold the old limit
   return GBI_OK;
 }
 

@@ -96,3 +96,31 @@ def test_scratch_that_moves_between_solves():
         for _ in range(3):
             _same(_solve(gbi, ctx, R, p, 1.0, trunc, 2), ref)
         ctx.close()
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+def test_wait_limit_of_a_replayed_solve(precision):
+    """gbi_set_wait_limit holds for later solves of captured sizes too: with no rounds every stage wait of
+    the tiled passes gives up, with the default restored the results are back."""
+    import torch
+    import paper_1411_0278_gb300 as gbi
+    R, p = _inputs(100, 8)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = gbi.Context(0, stream=stream)
+    ctx.set_wpt(1)
+    ref = _solve(gbi, ctx, R, p, 1.0, 2, precision, repeats=3)
+    i = ctx.trap_inputs(100, 2, 0.01, 0.1, 0.05, 0.02, R, p)
+    prm = gbi.params(a=1.0, eta=0.05, trunc=2, precision=precision, rtol=1e-10, max_iter=60, max_refine=3)
+    short = lambda: ctx.solve(prm, R, i["Va"], i["Oa"], i["VH"], i["Fe"], i["Te"], allow_not_converged=True)
+    for _ in range(3):
+        short()
+    ctx.set_wait_limit(0)
+    for _ in range(3):
+        with pytest.raises(gbi.GbiError) as err:
+            short()
+        assert err.value.status == gbi.GBI_ERR_TIMEOUT
+    ctx.set_wait_limit(-1)
+    for _ in range(3):
+        _same(_solve(gbi, ctx, R, p, 1.0, 2, precision), ref)
+    ctx.close()
