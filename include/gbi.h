@@ -492,7 +492,8 @@ gbi_status gbi_pass_status(gbi_ctx* ctx);
  * counted as launches; their few microseconds stay in the summed time.  Class ids:
  * precision * 9 + rows * 3 + cols for gbi_apply-style passes (precision 0 = FP64,
  * 1 = FP32, 2 = double-float; rows/cols 0 = all, 1 = rigid-body, 2 = higher),
- * 27 = closed-form trap pass in FP64, 28 = in FP32, 29 = flow field (gbi_flow) in FP64,
+ * 27 = closed-form trap pass in FP64, 28 = in FP32 (superposition steps of up to 72
+ * spheres: the launch that runs them all, up to 4096), 29 = flow field (gbi_flow) in FP64,
  * 30 = in FP32, 31 = wall images (gbi_wall_superpose) in FP64, 32 = in FP32 (flops: the closed
  * form per (target, source) term times N^2).  gbi_kernel_stats synchronizes
  * on the recorded events. */

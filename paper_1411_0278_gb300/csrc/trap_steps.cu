@@ -384,16 +384,17 @@ gbi_status run_steps(gbi_ctx* ctx, const StepPar& c, int nsteps, double* R, doub
   // the dipole 13 more
   const double flops = (DIP ? 116.0 : 103.0) * double(c.N) * double(c.N - 1);
   const int ns = trap_splits(c.N, 1), chunk = (c.N + ns - 1) / ns;   // at most 2 splits up to kStepsSmall
-  if (c.N <= kStepsSmall && !ctx->prof) {
+  if (c.N <= kStepsSmall) {
     const int half = (c.N * ns + 31) / 32 * 32;   // threads of one kind of sum
     const int threads = half + half > 4 * c.N ? half + half : (4 * c.N + 31) / 32 * 32;
-    // a launch stays below some ten milliseconds
+    // a launch stays below 40 ms (4096 steps of 72 spheres: 33)
     for (int done = 0; done < nsteps; done += 4096) {
-      k_steps_small<DIP><<<1, threads, 0, ctx->stream>>>(c, nsteps - done < 4096 ? nsteps - done : 4096, ns, chunk,
-                                                      half, R, p);
-      ++ctx->launches;
+      const int n = nsteps - done < 4096 ? nsteps - done : 4096;
+      GBI_CHECK(timed(ctx, 28, n * flops, 1, [&] {
+        k_steps_small<DIP><<<1, threads, 0, ctx->stream>>>(c, n, ns, chunk, half, R, p);
+        return cudaGetLastError();
+      }));
     }
-    GBI_CHECK(cudaGetLastError());
     return GBI_OK;
   }
   GBI_TRY(ensure(ctx, ctx->trapbuf, sizeof(float) * ((size_t)c.N * W + (size_t)ns * c.N * 6)));
