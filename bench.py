@@ -9,7 +9,7 @@ FP64 Arnoldi, iterative refinement to ||b - A q|| / ||b|| <= 1e-10, output pass)
 and one forward-Euler update, all inside libgbi.
 
 Metric: pair-interactions/s (ordered pairs summed over every pair pass of the
-step) and solves/s.  Also reported: the roofline of the dominant kernel, the
+step) and solves/s, in one printed line.  Also measured, and written to the details file: the roofline of the dominant kernel, the
 end-to-end number through the host-pointer C-ABI call, every precision mode of
 the same solve with its residual against the FP64 system, the N = 64 FP64
 trajectory (100 re-solved Euler steps), the N = 10^4 superposition trajectory
@@ -251,6 +251,36 @@ def run_reference(args):
                              "cpu_model": cpu_model()},
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
     print(json.dumps(line), flush=True)
+
+
+# what the printed line holds; the full record (every mode, secondary workload and trajectory, some
+# 30 KB) goes to the details file, because readers of the line keep only a few KB of output
+HEADLINE = ["metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "precision", "data", "config", "solves_per_s", "residual_vs_fp64_system", "roofline",
+            "cpu_baseline", "e2e", "clocks", "gpu_launches"]
+
+
+NOTES = {"roofline": ("traffic_note", "peak_source", "flop_convention", "timing"), "cpu_baseline": ("solve_N64_l2", "solve_N1024_l3", "superposition_N10000")}
+
+
+def headline(line):
+    """The printed part of the record, without the longer notes of its entries."""
+    out = {k: line[k] for k in HEADLINE if k in line}
+    for k, drop in NOTES.items():
+        if isinstance(out.get(k), dict):
+            out[k] = {q: v for q, v in out[k].items() if q not in drop}
+    return out
+
+
+def emit(line, details):
+    """The one printed line, and the full record in the file `details` (empty: not written)."""
+    if details:
+        try:
+            with open(details, "w") as f:
+                json.dump(line, f)
+        except OSError as e:
+            print("bench: details not written: %s" % e, file=sys.stderr)
+    print(json.dumps(headline(line)), flush=True)
 
 
 # passes timed by gbi_tune, in the order of its result
@@ -1125,7 +1155,7 @@ def run_ours(args):
                 "periodic_superposition": periodic_line, "flow_field": flowline, "config1_trajectory": traj64, "config3_trajectory": traj3,
                 "config3_paper_geometry": trajp, "squirmer_pair_orbits": pair_orbits, "batched": batched, "learned_nearfield": learned,
                 "tuned_wpt": dict(zip(TUNED_PASSES, tuned))}
-        print(json.dumps(line), flush=True)
+        emit(line, args.details)
     ctx.close()
     if world > 1:
         torch.distributed.destroy_process_group()
@@ -1140,6 +1170,8 @@ def main():
     ap.add_argument("--precision", type=int, default=3, choices=[0, 1, 2, 3],
                     help="0 all FP64; 1 FP32 GMRES + FP64 refinement; 2 FP32 GMRES + double-float refinement, "
                          "RHS and outputs; 3 as 2 with FP32 RHS and outputs")
+    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
+                    help="file for the full record (the printed line holds the headline numbers)")
     args = ap.parse_args()
     if args.impl == "reference":
         run_reference(args)
