@@ -351,7 +351,8 @@ gbi_status gbi_solve_static(void* stream, const gbi_params* params, int N,
  * (decided in FP64 as (dx dx + dy dy) + dz dz), grouped by n and sorted by m; systems
  * as in gbi_batch_solve (nsys <= 1 and offsets NULL: one system).  One system of more
  * than 4096 spheres uses a cell list and fails with GBI_ERR_ARG if a sphere has more
- * than 64 such neighbours.  *npairs receives the count; gbi_pairs_get copies the last
+ * than 64 such neighbours; its search keeps 256 bytes of workspace per sphere in the
+ * context.  *npairs receives the count; gbi_pairs_get copies the last
  * list into device arrays tg (targets n), sr (sources m) of *npairs ints.
  * Synchronizes the stream.
  * gbi_mlp_set / gbi_mlp_get: load (host FP32, resets Adam) / read the weights and the

@@ -83,7 +83,8 @@ size_t scan_scratch_ints(int n) { return (size_t)((n + 1023) / 1024) + 1; }
 
 // Up to this many counts one kernel scans: every block adds up all the counts before its own
 // chunk itself (L2 reads, at most 1 MB a block) instead of waiting for the other blocks or for
-// two more launches.  n = 10^5: one launch against three (9 us).
+// two more launches.  n = 10^5: one launch against three (9 us); at the limit neither form is ahead
+// (gbi_pairs N = 262144 / 262145: 137 / 137 us).
 constexpr int kScanOne = 1 << 18;
 
 __device__ __forceinline__ int block_sum_1024(int v, int* s_warp) {
@@ -267,7 +268,7 @@ __global__ void k_cell_fill(int N, const double* __restrict__ R, const int* __re
   rec[cell_start[cell_of[n]] + rank[n]] = make_float4(float(r[0]), float(r[1]), float(r[2]), __int_as_float(n));
 }
 
-constexpr int kMaxNb = 64;   // neighbours kept per sphere in the cell-list path
+constexpr int kMaxNb = 64;   // neighbours kept per sphere in the cell-list path (256 bytes of slots a sphere)
 
 // Neighbours of every sphere, in no particular order, into its row of kMaxNb slots, and their
 // number.  One thread per record in bucket order, so the lanes of a warp walk the same buckets
@@ -900,7 +901,9 @@ cudaError_t adam(float* th, float* m, float* v, const float* g, int t, double lr
 // neighbour-list driver
 // ---------------------------------------------------------------------------------
 
-// systems of this many spheres on average are scanned by a warp per target
+// Systems of this many spheres on average are scanned by a warp per target.  The line is not sharp: gbi_pairs
+// for 1000 systems of 12 / 15 by threads 74 / 72 us, of 16 / 20 by warps 73 / 79 (FP64 scans by threads: 220 / 221 / 223 /
+// 231); 100 of 100: 66 (158).
 constexpr int kNbWarpMean = 16;
 
 static cudaError_t nb_scan_systems(int N, const double* R, const int* sys_of, const int* sys_off, int nsys, double rc,
@@ -941,8 +944,11 @@ cudaError_t nb_search(int N, const double* R, double rc, double rc2, int* cell_o
   g.lx = (bits + 2) / 3;
   g.ly = (bits + 1) / 3;
   g.lz = bits / 3;
-  // the side exceeds rc by more than the rounding of x / side, so that spheres closer than rc
-  // are never two cells apart
+  // Spheres closer than rc are never two cells apart, wherever they are: the side exceeds rc, so
+  // their exact quotients x inv differ by less than 1; rounding is monotonic and every integer below 2^53
+  // is an FP64 number, so rounded quotients with an integer k between their floors, u1 < k and u2 >= k + 1,
+  // would need exact ones at least 1 apart.  (Beyond 2^53 cells from the origin neighbouring FP64
+  // coordinates are further apart than rc.)
   g.inv = 1.0 / (rc * (1.0 + 1.0 / 1048576.0));
   const int nc = 1 << bits;
   cudaError_t e = cudaMemsetAsync(cell_cnt, 0, sizeof(int) * nc, st);
