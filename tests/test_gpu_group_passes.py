@@ -124,3 +124,17 @@ def test_tuning_a_batch_of_small_systems(trunc, sizes):
     for x, y in zip(got, ref):
         close(x, y, 1e-8)
     ctx.close()
+
+
+def test_layout_follows_the_choice():
+    """A forced warps-per-target choice between calls changes kernels and vector layouts together."""
+    gbi, ctx, R, offs, a = _case(3, [2, 3] * 400)
+    prm = gbi.params(a=1.0, eta=0.7, trunc=3, precision=2, rtol=1e-10)
+    first = None
+    for w in (0, 0, 4, 4, 0, 8, 0):
+        ctx.set_wpt(w)
+        got = ctx.batch_solve(prm, offs, R, *a)[:3]
+        first = first or got
+        for x, y in zip(got, first):
+            close(x, y, 1e-8)
+    ctx.close()
