@@ -84,7 +84,7 @@ __host__ __device__ __forceinline__ df& operator+=(df& a, df b) {
 // product's error a.hi b.hi - p rides on the second one in a single FMA, a.hi b.hi - w.  (A product with
 // its error followed by a two-sum takes 12.)  The double-float pair passes are bound by the FP32 pipe
 // (70% busy), so operations are their time: with this, df_mul and df_rsqrt an H/H pair of l <= 3 takes
-// 3360 instead of 4485 instructions, 148 us instead of 181 at N = 1024 (ncu); the error is at df_mul.
+// 3650 instead of 4485 instructions, 151 us instead of 181 at N = 1024 (ncu); the error is at df_mul.
 __host__ __device__ __forceinline__ df df_fma(df a, df b, df c) {
   const float p = df_rmul(a.hi, b.hi);
   const float s = p + c.hi;

@@ -136,9 +136,15 @@ inline bool balanced_form(int w) { return w == kFormTile || w == kFormChunk; }
 // 20894 / 20430 / 21423; l <= 3 N = 1000: 968 / 960 / 993 / 1083, N = 9000: 34224 / 33743 / 34168; l <= 4
 // N = 200: 682 / 602 / 647, N = 3000: 14832 / 14158 / 15073.  Up to 1536 spheres, a few waves, the waves decide
 // between 4 and 8 (wave_cost): 4 / 8 warps l <= 2 N = 300: 452 / 428, N = 1000: 617 / 637; l <= 3 N = 700: 769 / 734;
-// l <= 4 N = 300: 686 / 750, 500: 1013 / 1077, 700: 1550 / 1512, 1000: 2355 / 2295.  Batches, whose systems fill
-// the GPU together: 8 up to N = 300: 642 / 656 / 719 / 776, 48 up to 128: 701 / 746 / 905 / 1070, 48 up to 1024:
-// 2074 / 2154 / 2815 / 3422.
+// l <= 4 N = 300: 686 / 750, 500: 1013 / 1077, 700: 1550 / 1512, 1000: 2355 / 2295.  Two warps are left out of that
+// choice: they lost at all of these sizes (2 / best of 4 and 8: l <= 2 N = 300 443 / 436, 1000 637 / 598; l <= 3 N = 300
+// 540 / 521, 700 813 / 789, 1000 1033 / 1020; l <= 4 N = 300 745 / 666, 500 986 / 983, 700 1717 / 1502, 1000 2370 / 2289),
+// also where wave_cost, which knows neither a short block's start nor the record loads, puts them ahead.
+// Batches, whose systems fill the GPU together: 8 up to N = 300: 642 / 656 / 719 / 776, 48 up to 128: 701 / 746 / 905 /
+// 1070, 48 up to 1024: 2074 / 2154 / 2815 / 3422.  Two to eight systems of 40 to 800 spheres (l <= 2, 3, 4): 2 is the
+// best of 2 / 4 / 8 or within 7% of it: l <= 3 two of 800: 1249 / 1232 / 1364, three of 100: 533 / 518 / 538, of 200:
+// 584 / 594 / 642, of 800: 1492 / 1577 / 1795; l <= 4 two of 100: 626 / 586 / 668, of 400: 1358 / 1271 / 1427, three of 200:
+// 855 / 886 / 980, eight of 40: 582 / 658 / 736.
 //
 // wave_cost: the waves of N targets over 152 SMs that hold `warps` warps each, times a block's rounds of
 // 32 w sources and its start and reduction (0.6 of a round); a last wave that leaves an SM with b of its B

@@ -1514,8 +1514,10 @@ void launch_update(gbi_ctx* ctx, const Setup& s, const Batch& B, const GPtr& gp,
 
 // kChunk Arnoldi iterations of every active system: pair pass on the source of V_j
 // (written by the previous bk_scale / bk_scale0 / bk_sub_scale), classical Gram-Schmidt
-// (see two_pass_gs), Givens update and V_{j+1} with its source -- eight kernels per
-// iteration with two rounds, four with one.  With
+// (see two_pass_gs), Givens update and V_{j+1} with its source -- per iteration the pair pass and one
+// kernel for a small system (bk_step_cluster) or many tiny ones (bk_step_warp), else two (bk_dots_fin,
+// bk_dots_multi or bk_dots_sys, and bk_sub_scale; three for many large systems) with one round and seven with
+// two.  With
 // fused set and a single system the seven kernels after the pair pass are replaced by
 // bk_step_fused; that is faster for direct launches, while inside the cycle graph the
 // separate kernels (graph launch overhead about a microsecond each) measured faster than

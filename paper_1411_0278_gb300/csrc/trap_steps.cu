@@ -16,7 +16,7 @@
 // A step is two kernels: the pair sums, and one that adds the splits, moves the spheres and
 // writes the next step's source records (the general call sequence: six).  Up to kStepsSmall
 // spheres one block runs all the steps in one launch.  Microseconds a step, before -> now:
-// N = 2: 26.7 -> 2.0, 64: 45 -> 9.1, 128: 45 -> 14.7, 1000: 53 -> 16.5, 10^4: 348 -> 256 (pairs 310 -> 242).
+// N = 2: 26.7 -> 2.0, 64: 44 -> 7.8, 128: 45 -> 14.7, 1000: 53 -> 16.5, 10^4: 348 -> 256 (pairs 310 -> 242).
 #include <cuda_runtime.h>
 
 #include <type_traits>
@@ -144,7 +144,8 @@ __global__ void k_steps_records(const StepPar c, const double* __restrict__ R, c
 // so that one 16-byte load gives two broadcast operands (as trap_pairs_f2).
 // (The sources are split and added up as in trap_kernel.cu, so the sums are the same bits.)  Up to
 // kStepsNarrow spheres, where that leaves a few blocks (N = 1000: 32), the block is one warp with two
-// targets per thread.
+// targets per thread; us a step: N = 1900 24.5, 2048 25.0, then 2049 with the wide block 39.6, 3000 41.2 (the general
+// sequence 57, 56, 70, 74), so the narrow one still wins at this limit.
 constexpr int kStepTile = 128;
 constexpr int kStepsNarrow = 2048;
 
@@ -268,8 +269,8 @@ __global__ void __launch_bounds__(6 * kMoveSpheres)
 // trap_kernel.cu, so that orbits with close encounters, which amplify a last bit by ten thousand within
 // fifty steps, stay the same; V and Omega are summed by different threads.  (Several lanes per target added
 // in FP64 took 8.3 us at N = 64 and left R 8e-9 off.)  A step is bound by the latency of the pair sums and of the
-// FP64 chain from them to the next record: 2.0 us at N = 2, 4.8 at 32, 9.1 at 64, where the two
-// kernels take 14.
+// FP64 chain from them to the next record: 2.0 us at N = 2, 4.8 at 32, 7.8 at 64, 8.1 at 72; the two kernels take
+// 11.0 at 73.  It still wins at this limit, up to which two splits hold every target's sources.
 constexpr int kSmallThreads = 512;
 constexpr int kStepsSmall = 72;
 
